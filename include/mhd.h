@@ -59,13 +59,15 @@ typedef enum {
 } mhd_status;
 
 typedef enum {
-  MHD_FP64 = 0,       /* IEEE double everywhere */
+  MHD_FP64 = 0,       /* IEEE double data, grid products and updates; each 1D transform in 64-bit
+                         fixed point with the pencil's own exponent, which rounds less than IEEE
+                         double arithmetic (a pencil with a NaN or an infinity gives NaNs) */
   MHD_FP32_MIXED = 1, /* FFT passes, grid products and the RHS assembly in FP32; the state kept
                          as a double-float pair of FP32 arrays (hi + lo, a 48-bit significand)
                          and advanced with an error-free two-sum; history and RK stage states in
                          FP32; dt computed in FP64 (from an FP32 CFL maximum); the k = 0 modes,
                          whose RHS is exactly zero, held exactly; diagnostics, spectra and
-                         set/get of the state in FP64 */
+                         set/get of the state in FP64 (the set in IEEE arithmetic throughout) */
   MHD_FP64_DF = 2     /* FP64-tolerance mode without FP64 arithmetic in the step: every value of
                          the step -- state, history, stage state, the intermediate spectra and the
                          grid products -- is a double-float pair (hi + lo FP32, a 48-bit

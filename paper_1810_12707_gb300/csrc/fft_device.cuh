@@ -7,6 +7,7 @@
 #pragma once
 
 #include "dfloat.cuh"
+#include "fixed64.cuh"
 #include "mhd_internal.h"
 
 #include <type_traits>
@@ -247,6 +248,13 @@ __device__ __forceinline__ cplx64 tw_load(const cplx64 *p) {
   asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.re), "=d"(v.im) : "l"(p));
   return v;
 }
+__device__ __forceinline__ TwFx tw_load(const TwFx *p) {
+  TwFx v;
+  asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.ch), "=r"(v.cl), "=r"(v.sh), "=r"(v.sl)
+               : "l"(p));
+  return v;
+}
 __device__ __forceinline__ cplx32 tw_load(const cplx32 *p) {
   cplx32 v;
   asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.re), "=f"(v.im) : "l"(p));
@@ -294,9 +302,13 @@ __device__ __forceinline__ void group_sync() {
   }
 }
 
-// ---- FP64 twiddles in FMA form ----
-// On GB300 the FP64 pipe bounds the FP64 transforms, so their twiddled stages use fewer FP64
-// instructions: every twiddle is kept as W = i^q c (1 + i t) with |t| <= 1, and a radix-2
+// ---- IEEE FP64 transforms: twiddles in FMA form ----
+// Only the transform of a mixed-precision initial state still runs in IEEE FP64 arithmetic (tables
+// of cplx64; every other FP64 transform takes a TwFx table and runs in fixed point, 2.5 to 3.1
+// times faster).  The mixed mode's FP32 steps turn a difference of 1e-17 in the state's smallest
+// modes into FP32 rounding noise within a step, so a faster transform here would change every
+// mixed trajectory by about 4e-8 (measured: 3.8e-8 after 60 steps at 32^3), no less exactly but
+// not reproducibly.  Its cost is FP64 instructions, so the twiddled stages use few: every twiddle is kept as W = i^q c (1 + i t) with |t| <= 1, and a radix-2
 // butterfly (a + W x, a - W x) costs six fused multiply-adds: z = x + i t x (two), z' = i^q z (an
 // exact swap and sign change done with integer operations), a +- c z' (four).  The table follows
 // the classic one in the same allocation: tw[0..N) classic W_N^m, then N pairs (c, t), then N
@@ -385,11 +397,11 @@ __device__ __forceinline__ void dft_twiddled_fma(cplx64 *v, int m, const cplx64 
   }
 }
 
-// The first (untwiddled) radix-8 stage in the same radix-2 layer form: twiddle 1 everywhere
-// except the quarter turns (free) and w8 = c (1 + i DIR), c = sqrt(2)/2, on two butterflies of
-// layer 3 (two additions and four FMAs each): 52 FP64 instructions instead of 56.  With ZP the
-// inputs 3 and 4 are known zeros (zero-padded inverse transforms: the 2/3-rule gap K+1 .. N-K-1
-// always covers them, see pencil_fft) and layer 1 loses two butterflies: 44.
+// The first (untwiddled) radix-8 stage as radix-2 layers: twiddle 1 everywhere except the quarter
+// turns (free) and w8 = c (1 + i DIR), c = sqrt(2)/2, on two butterflies of layer 3 (two additions
+// and four FMAs each).  With ZP the inputs 3 and 4 are known zeros (zero-padded inverse
+// transforms: the 2/3-rule gap K+1 .. N-K-1 always covers them, see pencil_fft) and layer 1 loses
+// two butterflies.
 template <int DIR, bool ZP, typename C>
 __device__ __forceinline__ void dft8_first_fma(C *v) {
   using R = typename C::value_type;
@@ -453,8 +465,8 @@ __device__ __forceinline__ void dft8_first_fma(cdf *v) {
 
 // ---- values per thread ----
 // FP32 pencils: 16 values per thread (radix 16: two shared-memory stages at N = 256 where radix 8
-// needs three; the FP32 passes are bound by instruction issue).  FP64: 8 (their cost is FP64
-// instructions, which radix 16 does not reduce).  A pencil is transformed by N / VPT threads.
+// needs three; the FP32 passes are bound by instruction issue).  FP64 and double-float: 8 (their
+// 16-byte values fill the registers).  A pencil is transformed by N / VPT threads.
 // Kernels may choose 8 or 16 for FP32 (the radix that suits a pass depends on N and on the pass;
 // the column passes let the autotuner pick); FP64 always uses 8.
 template <typename C>
@@ -487,7 +499,7 @@ __device__ __forceinline__ void stockham_stages(C *buf, int t, bool active, cons
     constexpr int NB = VPT / R;
     constexpr int TPP = tpp_for<N, VPT>();
     constexpr int TWSTEP = N / (NS * R);
-    // FP64 stages with twiddles take them inside the butterflies (FMA form, fewer FP64
+    // IEEE FP64 stages with twiddles take them inside the butterflies (FMA form, fewer FP64
     // instructions); the others multiply on load.
     constexpr bool kFma = std::is_same<C, cplx64>::value && NS > 1;
     // The first radix-8 stage: FMA layers, and with ZP the zero inputs 3 and 4 skipped; the first
@@ -546,13 +558,148 @@ __device__ __forceinline__ void stockham_stages(C *buf, int t, bool active, cons
   }
 }
 
+// ---- The FP64 pencil FFT (fixed64.cuh) ----
+// The same Stockham stages on a pencil of doubles.  The first stage reads doubles, finds the
+// pencil's common exponent and converts; the pencil is fixed-point complex values between the
+// stages; the last stage writes doubles.  Against the IEEE FP64 stages this replaced (FP64 pipe 92 %
+// busy), ms per pass: 512^3 inverse y 12.4 -> 4.13, forward y 23.8 -> 8.54, flux 65.6 -> 27.0;
+// 256^3 step 14.75 -> 5.38.  The exponent's reduction adds no barrier: a group of
+// more than a warp leaves its warps' parts in shared memory before the barrier that the first
+// stage has between its reads and its writes anyway.  It depends on the group's threads only, so
+// a pencil's results are the same bits in every kernel and at every tile width.
+template <int N, int DIR, int NS>
+__device__ __forceinline__ void fx_stages(cfx *buf, int t, bool active, const TwFx *__restrict__ tw, const FxScale &sc,
+                                          int left) {
+  constexpr int R = N / NS >= 8 ? 8 : N / NS;
+  constexpr int NB = 8 / R;
+  constexpr int TPP = tpp_for<N, 8>();
+  constexpr int TWSTEP = N / (NS * R);
+  constexpr int LOG2R = R == 8 ? 3 : R == 4 ? 2 : 1;
+  const int s = left < LOG2R ? left : LOG2R;  // this stage's right shift
+  cfx v[8];
+  if (active) {
+    const TwFx *ts = tw + s * N;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const int j = t + b * TPP;
+      const int k = j % NS;
+      v[b * R] = fx_shift(buf[sm_idx<cplx64>(j)], s);
+#pragma unroll
+      for (int r = 1; r < R; ++r)
+        v[b * R + r] = fx_mul<DIR>(buf[sm_idx<cplx64>(j + r * (N / R))], tw_load(ts + r * k * TWSTEP));
+      fx_dft<R, DIR>(v + b * R);
+    }
+  }
+  group_sync<TPP>();
+  if (active) {
+    const uint32_t be = sc.ek + (uint32_t)sc.shift + 1u;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const int j = t + b * TPP;
+      const int base = (j / NS) * NS * R + j % NS;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const cfx x = v[b * R + r];
+        cfx *p = buf + sm_idx<cplx64>(base + r * NS);
+        if constexpr (NS * R < N) {
+          *p = x;
+        } else {
+          cplx64 d = {fx_to_double(x.re, be), fx_to_double(x.im, be)};
+          if (sc.bad) d.re = d.im = fx_double(0x7ff80000u, 0u);
+          *reinterpret_cast<cplx64 *>(p) = d;
+        }
+      }
+    }
+  }
+  group_sync<TPP>();
+  if constexpr (NS * R < N) fx_stages<N, DIR, NS * R>(buf, t, active, tw, sc, left - s);
+}
+
+template <int N, int DIR, bool ZP>
+__device__ __forceinline__ void fx_pencil_fft(cplx64 *buf, int t, bool active, const TwFx *__restrict__ tw) {
+  constexpr int TPP = tpp_for<N, 8>();
+  constexpr int LOG2G = TPP == 128 ? 7 : TPP == 64 ? 6 : TPP == 32 ? 5 : TPP == 16 ? 4 : TPP == 8 ? 3 : TPP == 4 ? 2 : 1;
+  constexpr int K = (N - 1) / 3;
+  static_assert(!ZP || (3 * (N / 8) > K && 5 * (N / 8) - 1 < N - K),
+                "inputs 3 and 4 of the first stage must lie in the 2/3-rule gap");
+  __shared__ FxPart part[32];  // one entry per warp, for groups of more than one
+  cplx64 x[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    x[r] = cplx64{0.0, 0.0};
+    if (!(ZP && (r == 3 || r == 4)) && active) x[r] = buf[sm_idx<cplx64>(t + r * TPP)];
+  }
+  uint32_t m = 0u;
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    if (ZP && (r == 3 || r == 4)) continue;
+    m = max(m, max(fx_hi(x[r].re) & 0x7fffffffu, fx_hi(x[r].im) & 0x7fffffffu));
+  }
+  m >>= 20;
+  if constexpr (TPP >= 32) {
+    m = __reduce_max_sync(0xffffffffu, m);
+  } else {
+#pragma unroll
+    for (int o = TPP / 2; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(existing_lanes(), m, o));
+  }
+  FxPart p = {m, 0u, 0u};
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    if (ZP && (r == 3 || r == 4)) continue;
+    p.a += fx_size(fx_hi(x[r].re), m) + fx_size(fx_hi(x[r].im), m);
+  }
+  p.t = (p.a >> 3) + 1u;
+  if constexpr (TPP >= 32) {
+    p.a = __reduce_max_sync(0xffffffffu, p.a);
+    p.t = __reduce_add_sync(0xffffffffu, p.t);
+  } else {
+#pragma unroll
+    for (int o = TPP / 2; o > 0; o >>= 1) {
+      p.a = max(p.a, __shfl_xor_sync(existing_lanes(), p.a, o));
+      p.t += __shfl_xor_sync(existing_lanes(), p.t, o);
+    }
+  }
+  if constexpr (TPP > 32) {
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = p;
+  }
+  group_sync<TPP>();
+  if constexpr (TPP > 32) {
+    const int w0 = (threadIdx.x / TPP) * (TPP / 32);
+    p = part[w0];
+#pragma unroll
+    for (int i = 1; i < TPP / 32; ++i) p = fx_merge(p, part[w0 + i]);
+  }
+  const FxScale sc = fx_scale(p, LOG2G);
+  cfx *fb = reinterpret_cast<cfx *>(buf);
+  if (active) {
+    cfx v[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      if (ZP && (r == 3 || r == 4)) continue;
+      v[r] = cfx{fx_from_double(fx_hi(x[r].re), fx_lo(x[r].re), sc.ek),
+                 fx_from_double(fx_hi(x[r].im), fx_lo(x[r].im), sc.ek)};
+    }
+    fx_dft8<DIR, ZP>(v);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) fb[sm_idx<cplx64>(8 * t + r)] = v[r];
+  }
+  group_sync<TPP>();
+  fx_stages<N, DIR, 8>(fb, t, active, tw, sc, sc.shift);
+}
+
 // `t` in [0, N / VPT): the thread's index within its pencil's group.  ZP: the pencil is
 // zero-padded by the 2/3 rule (elements K+1 .. N-K-1 are zero, K = (N-1)/3), as every inverse
 // transform of a truncated spectrum is; the FP64 first stage then skips the inputs it knows are
 // zero (they need not even be written).
-template <int N, int DIR, typename C, int VPT = fft_vpt<C>(), bool ZP = false, bool TWG = false>
-__device__ __forceinline__ void pencil_fft(C *buf, int t, bool active, const C *__restrict__ tw) {
-  stockham_stages<N, DIR, 1, C, VPT, ZP, TWG>(buf, t, active, tw);
+// TW: the twiddle table's type; a TwFx table runs an FP64 pencil in fixed point.
+template <int N, int DIR, typename C, int VPT = fft_vpt<C>(), bool ZP = false, bool TWG = false, typename TW>
+__device__ __forceinline__ void pencil_fft(C *buf, int t, bool active, const TW *__restrict__ tw) {
+  if constexpr (std::is_same<TW, TwFx>::value) {
+    static_assert(std::is_same<C, cplx64>::value && VPT == 8, "fixed-point transforms are FP64's, radix 8");
+    fx_pencil_fft<N, DIR, ZP>(buf, t, active, tw);
+  } else {
+    stockham_stages<N, DIR, 1, C, VPT, ZP, TWG>(buf, t, active, tw);
+  }
 }
 
 // FFT index of kept index j (0..2K) along a truncated axis: j for j <= K, else j - (2K+1) + N.

@@ -31,10 +31,10 @@ constexpr size_t tws_bytes() { return tws_staged<CC, N>() ? (size_t)N * sizeof(C
 // row (coalesced) and no index needs a division.
 // VPT: values per thread of the transform (8, or 16 for FP32), so N / VPT threads per column.
 // One tile (TC columns of one slab): work item w = slab * ntiles + tile.
-template <int N, int DIR, typename CI, typename CO, typename CC, int VPT>
+template <int N, int DIR, typename CI, typename CO, typename CC, int VPT, typename TW>
 __device__ __forceinline__ void col_fft_tile(const CI *__restrict__ in, CO *__restrict__ out, unsigned w, int ntiles,
                                              int tsh, int cols, typename scale_of<CC>::type scale,
-                                             const CC *__restrict__ tw, CC *sm) {
+                                             const TW *__restrict__ tw, CC *sm) {
   constexpr int TPP = tpp_for<N, VPT>();
   constexpr int P = pencil_pitch<CC>(N);
   constexpr int K = (N - 1) / 3;  // the 2/3-rule cut-off, fixed by N
@@ -71,7 +71,7 @@ __device__ __forceinline__ void col_fft_tile(const CI *__restrict__ in, CO *__re
   }
   // double-float at N >= 512: the twiddle table staged in shared memory behind the pencils
   constexpr bool kTws = tws_staged<CC, N>();
-  const CC *twp = tw;
+  const TW *twp = tw;
   if constexpr (kTws) {
     CC *tws = sm + tc * P;
     for (int i = threadIdx.x; i < N; i += blockDim.x) tws[i] = tw[i];
@@ -95,41 +95,41 @@ __device__ __forceinline__ void col_fft_tile(const CI *__restrict__ in, CO *__re
   }
 }
 
-template <int N, int DIR, typename CI, typename CO, typename CC, int VPT>
+template <int N, int DIR, typename CI, typename CO, typename CC, int VPT, typename TW>
 __global__ void col_fft_kernel(const CI *__restrict__ in, CO *__restrict__ out, int ntiles, int tsh,
-                               int cols, typename scale_of<CC>::type scale, const CC *__restrict__ tw) {
+                               int cols, typename scale_of<CC>::type scale, const TW *__restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  col_fft_tile<N, DIR, CI, CO, CC, VPT>(in, out, blockIdx.x, ntiles, tsh, cols, scale, tw,
+  col_fft_tile<N, DIR, CI, CO, CC, VPT, TW>(in, out, blockIdx.x, ntiles, tsh, cols, scale, tw,
                                         reinterpret_cast<CC *>(smem_raw));
 }
 
 // Double-float forward passes: the same tile with 4 blocks of 256 threads per SM (64 registers a
 // thread), which measured 8 % faster at 512^3 than the 3 blocks that 72 registers allow (the
 // inverse passes measured slower so and keep col_fft_kernel).
-template <int N, int DIR, typename CI, typename CO, typename CC, int VPT>
+template <int N, int DIR, typename CI, typename CO, typename CC, int VPT, typename TW>
 __global__ void __launch_bounds__(256, 4) col_fft_kernel_b4(const CI *__restrict__ in, CO *__restrict__ out,
                                                            int ntiles, int tsh, int cols,
                                                            typename scale_of<CC>::type scale,
-                                                           const CC *__restrict__ tw) {
+                                                           const TW *__restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  col_fft_tile<N, DIR, CI, CO, CC, VPT>(in, out, blockIdx.x, ntiles, tsh, cols, scale, tw,
+  col_fft_tile<N, DIR, CI, CO, CC, VPT, TW>(in, out, blockIdx.x, ntiles, tsh, cols, scale, tw,
                                         reinterpret_cast<CC *>(smem_raw));
 }
 
 // The kernel a pass launches.
-template <int N, int DIR, typename CI, typename CO, int VPT>
+template <int N, int DIR, typename CI, typename CO, int VPT, typename TW = typename tw_of<CO>::type>
 constexpr auto col_kernel() {
-  if constexpr (std::is_same<CO, cdf>::value && DIR < 0) return col_fft_kernel_b4<N, DIR, CI, CO, CO, VPT>;
-  else return col_fft_kernel<N, DIR, CI, CO, CO, VPT>;
+  if constexpr (std::is_same<CO, cdf>::value && DIR < 0) return col_fft_kernel_b4<N, DIR, CI, CO, CO, VPT, TW>;
+  else return col_fft_kernel<N, DIR, CI, CO, CO, VPT, TW>;
 }
 
 // The same pass as a persistent kernel: a grid of (SMs x resident blocks) takes tiles from the
 // work counter ctr[0] until all `total` are done; ctr[1] counts the blocks that have finished, and
 // the last one resets both for the next launch (every block has taken its last tile by then; no
 // block waits on another).  Each tile's arithmetic is the one col_fft_kernel does.
-template <int N, int DIR, typename CI, typename CO, typename CC, int VPT>
+template <int N, int DIR, typename CI, typename CO, typename CC, int VPT, typename TW>
 __global__ void col_fft_persistent_kernel(const CI *__restrict__ in, CO *__restrict__ out, int ntiles, int tsh,
-                                          int cols, typename scale_of<CC>::type scale, const CC *__restrict__ tw,
+                                          int cols, typename scale_of<CC>::type scale, const TW *__restrict__ tw,
                                           unsigned total, unsigned *ctr) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned next;
@@ -138,7 +138,7 @@ __global__ void col_fft_persistent_kernel(const CI *__restrict__ in, CO *__restr
     __syncthreads();
     const unsigned w = next;
     if (w >= total) break;
-    col_fft_tile<N, DIR, CI, CO, CC, VPT>(in, out, w, ntiles, tsh, cols, scale, tw, reinterpret_cast<CC *>(smem_raw));
+    col_fft_tile<N, DIR, CI, CO, CC, VPT, TW>(in, out, w, ntiles, tsh, cols, scale, tw, reinterpret_cast<CC *>(smem_raw));
     __syncthreads();  // the tile's shared memory and `next` are free again
   }
   if (threadIdx.x == 0) {
@@ -172,12 +172,12 @@ int floor_log2(int v) {
 }
 
 // Largest thread count a launch of this instantiation may use (its registers bound it below 1024).
-template <int N, int DIR, typename CI, typename CO, int VPT>
+template <int N, int DIR, typename CI, typename CO, int VPT, typename TW = typename tw_of<CO>::type>
 int col_max_threads() {
   static int cached = 0;
   if (cached == 0) {
     cudaFuncAttributes a;
-    cached = cudaFuncGetAttributes(&a, col_kernel<N, DIR, CI, CO, VPT>()) == cudaSuccess ? a.maxThreadsPerBlock
+    cached = cudaFuncGetAttributes(&a, col_kernel<N, DIR, CI, CO, VPT, TW>()) == cudaSuccess ? a.maxThreadsPerBlock
                                                                                                : 256;
   }
   return cached;
@@ -211,12 +211,12 @@ int sm_count() {
   return sms;
 }
 
-template <int N, int DIR, typename CI, typename CO, int VPT>
-cudaError_t launch_col_v(const CI *in, CO *out, int nslab, int cols, double scale, const CO *tw,
+template <int N, int DIR, typename CI, typename CO, int VPT, typename TW = typename tw_of<CO>::type>
+cudaError_t launch_col_v(const CI *in, CO *out, int nslab, int cols, double scale, const TW *tw,
                          cudaStream_t s, int tile, unsigned *ctr) {
   constexpr int TPP = tpp_for<N, VPT>();
   int tc = tile > 0 ? tile : pick_tc(TPP, cols, sizeof(CO));
-  const int max_threads = col_max_threads<N, DIR, CI, CO, VPT>();
+  const int max_threads = col_max_threads<N, DIR, CI, CO, VPT, TW>();
   while (tc > 1 && tc * TPP > max_threads) tc /= 2;
   if (tc < 1) tc = 1;
   const int tsh = floor_log2(tc);  // a requested width that is not a power of two is rounded down
@@ -227,7 +227,7 @@ cudaError_t launch_col_v(const CI *in, CO *out, int nslab, int cols, double scal
   if (blocks <= 0) return cudaSuccess;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   if (ctr != nullptr) {
-    constexpr auto kfn = col_fft_persistent_kernel<N, DIR, CI, CO, CO, VPT>;
+    constexpr auto kfn = col_fft_persistent_kernel<N, DIR, CI, CO, CO, VPT, TW>;
     if (smem > 48 * 1024) {
       cudaError_t e = ensure_smem<kfn>((int)smem);
       if (e != cudaSuccess) return e;
@@ -239,28 +239,28 @@ cudaError_t launch_col_v(const CI *in, CO *out, int nslab, int cols, double scal
     return cudaGetLastError();
   }
   if (smem > 48 * 1024) {
-    cudaError_t e = ensure_smem<col_kernel<N, DIR, CI, CO, VPT>()>((int)smem);
+    cudaError_t e = ensure_smem<col_kernel<N, DIR, CI, CO, VPT, TW>()>((int)smem);
     if (e != cudaSuccess) return e;
   }
-  col_kernel<N, DIR, CI, CO, VPT>()<<<(unsigned)blocks, tc * TPP, smem, s>>>(
+  col_kernel<N, DIR, CI, CO, VPT, TW>()<<<(unsigned)blocks, tc * TPP, smem, s>>>(
       in, out, ntiles, tsh, cols, (typename scale_of<CO>::type)scale, tw);
   return cudaGetLastError();
 }
 
 // Radix of a column pass: `vpt` 8 or 16 (FP32 only); 0 picks the library default (radix 8, and
 // radix 16 for FP32 at N >= 512, where it measured faster).
-template <int N, int DIR, typename CI, typename CO>
-cudaError_t launch_col_n(const CI *in, CO *out, int nslab, int cols, double scale, const CO *tw,
+template <int N, int DIR, typename CI, typename CO, typename TW>
+cudaError_t launch_col_n(const CI *in, CO *out, int nslab, int cols, double scale, const TW *tw,
                          cudaStream_t s, int tile, int vpt, unsigned *ctr) {
   if constexpr (sizeof(CO) == 8) {
     if (vpt == 16 || (vpt == 0 && N >= 512))
-      return launch_col_v<N, DIR, CI, CO, 16>(in, out, nslab, cols, scale, tw, s, tile, ctr);
+      return launch_col_v<N, DIR, CI, CO, 16, TW>(in, out, nslab, cols, scale, tw, s, tile, ctr);
   }
-  return launch_col_v<N, DIR, CI, CO, 8>(in, out, nslab, cols, scale, tw, s, tile, ctr);
+  return launch_col_v<N, DIR, CI, CO, 8, TW>(in, out, nslab, cols, scale, tw, s, tile, ctr);
 }
 
-template <int DIR, typename CI, typename CO>
-cudaError_t launch_col(const CI *in, CO *out, int n, int nslab, int cols, double scale, const CO *tw,
+template <int DIR, typename CI, typename CO, typename TW>
+cudaError_t launch_col(const CI *in, CO *out, int n, int nslab, int cols, double scale, const TW *tw,
                        cudaStream_t s, int tile, int vpt, unsigned *ctr = nullptr) {
   switch (n) {
     case 16: return launch_col_n<16, DIR>(in, out, nslab, cols, scale, tw, s, tile, vpt, ctr);
@@ -323,7 +323,7 @@ int col_max_tile(int n, int dir, bool fp64, bool mixed_in, int vpt) {
 }
 
 cudaError_t launch_col_inverse(const cplx64 *in, cplx64 *out, int n, int nslab, int cols,
-                               const cplx64 *tw, cudaStream_t s, int tile, int, unsigned *ctr) {
+                               const TwFx *tw, cudaStream_t s, int tile, int, unsigned *ctr) {
   return launch_col<+1>(in, out, n, nslab, cols, 1.0, tw, s, tile, 8, ctr);
 }
 cudaError_t launch_col_inverse(const cplx64 *in, cplx32 *out, int n, int nslab, int cols,
@@ -335,8 +335,12 @@ cudaError_t launch_col_inverse(const cplx32 *in, cplx32 *out, int n, int nslab, 
   return launch_col<+1>(in, out, n, nslab, cols, 1.0, tw, s, tile, vpt, ctr);
 }
 cudaError_t launch_col_forward(const cplx64 *in, cplx64 *out, int n, int nslab, int cols,
-                               double scale, const cplx64 *tw, cudaStream_t s, int tile, int, unsigned *ctr) {
+                               double scale, const TwFx *tw, cudaStream_t s, int tile, int, unsigned *ctr) {
   return launch_col<-1>(in, out, n, nslab, cols, scale, tw, s, tile, 8, ctr);
+}
+cudaError_t launch_col_forward(const cplx64 *in, cplx64 *out, int n, int nslab, int cols,
+                               double scale, const cplx64 *tw, cudaStream_t s) {
+  return launch_col<-1>(in, out, n, nslab, cols, scale, tw, s, 0, 8);
 }
 cudaError_t launch_col_forward(const cplx32 *in, cplx32 *out, int n, int nslab, int cols,
                                double scale, const cplx32 *tw, cudaStream_t s, int tile, int vpt, unsigned *ctr) {

@@ -28,7 +28,7 @@ constexpr int threads_for(int tpp, int pencils) {
 }
 
 template <int N, int DIR, typename Ptr>
-__device__ __forceinline__ void fft_pencils(int np, Ptr ptr, const cplx64 *__restrict__ tw) {
+__device__ __forceinline__ void fft_pencils(int np, Ptr ptr, const TwFx *__restrict__ tw) {
   constexpr int TPP = tpp_for<N, 8>();
   const int G = blockDim.x / TPP;
   const int g = threadIdx.x / TPP, t = threadIdx.x - g * TPP;
@@ -48,7 +48,7 @@ __device__ __forceinline__ void fft_pencils(int np, Ptr ptr, const cplx64 *__res
 template <int N>
 __global__ void __launch_bounds__(kMaxThreads) velocity_x_kernel(const cplx64 *__restrict__ in,
                                                                   cplx64 *__restrict__ out, int K,
-                                                                  const cplx64 *__restrict__ tw) {
+                                                                  const TwFx *__restrict__ tw) {
   constexpr int KT = (N - 1) / 3;  // the 2/3-rule cut-off, fixed by N
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx64 *sm = reinterpret_cast<cplx64 *>(smem_raw);
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(256) absmax_kernel(const double *__restrict__ 
 namespace {
 
 template <int N>
-cudaError_t velocity_n(const cplx64 *in, cplx64 *out, const Dims &d, const cplx64 *tw, cudaStream_t s) {
+cudaError_t velocity_n(const cplx64 *in, cplx64 *out, const Dims &d, const TwFx *tw, cudaStream_t s) {
   constexpr int PAIRS = pairs_for(N);
   const int blocks = N * N / (2 * PAIRS);
   const int threads = threads_for(tpp_for<N, 8>(), 4 * PAIRS);
@@ -224,7 +224,7 @@ int num_shells(int k) {
   return s + 1;
 }
 
-cudaError_t launch_velocity_x(const cplx64 *in, cplx64 *out, const Dims &d, const cplx64 *tw, cudaStream_t s) {
+cudaError_t launch_velocity_x(const cplx64 *in, cplx64 *out, const Dims &d, const TwFx *tw, cudaStream_t s) {
   switch (d.n) {
     case 16: return velocity_n<16>(in, out, d, tw, s);
     case 32: return velocity_n<32>(in, out, d, tw, s);

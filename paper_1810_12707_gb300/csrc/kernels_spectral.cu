@@ -806,7 +806,7 @@ __global__ void __launch_bounds__(fused_max_threads<N, VPT>(), (fused_max_thread
     assemble_iz_kernel(const C *__restrict__ flux, C *state, C *lo, C *__restrict__ hist,
                        const PhysDev *__restrict__ phys, const StepCoef *__restrict__ coef,
                        const C *__restrict__ force, C *__restrict__ z_out, int tsh,
-                       typename scale_of<C>::type inv_n3, const C *__restrict__ tw) {
+                       typename scale_of<C>::type inv_n3, const typename tw_of<C>::type *__restrict__ tw) {
   constexpr int TPP = tpp_for<N, VPT>();
   constexpr int P = pencil_pitch<C>(N);
   constexpr int K = (N - 1) / 3;
@@ -866,7 +866,7 @@ namespace {
 
 template <int N, int VPT, typename C>
 cudaError_t assemble_iz_n(const C *flux, C *state, C *lo, C *hist, const PhysDev *phys, const StepCoef *coef,
-                          const C *force, C *z_out, const C *tw, int nb, int tile, cudaStream_t s) {
+                          const C *force, C *z_out, const typename tw_of<C>::type *tw, int nb, int tile, cudaStream_t s) {
   constexpr int TPP = tpp_for<N, VPT>();
   constexpr int K = (N - 1) / 3;
   constexpr int COLS = (2 * K + 1) * (K + 1);
@@ -894,7 +894,7 @@ cudaError_t assemble_iz_n(const C *flux, C *state, C *lo, C *hist, const PhysDev
 
 template <int VPT, typename C>
 cudaError_t assemble_iz_v(const C *flux, C *state, C *lo, C *hist, const PhysDev *phys, const StepCoef *coef,
-                          const C *force, C *z_out, const C *tw, const Dims &d, int tile, cudaStream_t s) {
+                          const C *force, C *z_out, const typename tw_of<C>::type *tw, const Dims &d, int tile, cudaStream_t s) {
   switch (d.n) {
     case 16: return assemble_iz_n<16, VPT>(flux, state, lo, hist, phys, coef, force, z_out, tw, d.batch, tile, s);
     case 32: return assemble_iz_n<32, VPT>(flux, state, lo, hist, phys, coef, force, z_out, tw, d.batch, tile, s);
@@ -910,7 +910,7 @@ cudaError_t assemble_iz_v(const C *flux, C *state, C *lo, C *hist, const PhysDev
 }  // namespace
 
 cudaError_t launch_assemble_iz(const cplx64 *flux, cplx64 *state, cplx64 *hist, const PhysDev *phys,
-                               const StepCoef *coef, const cplx64 *force, cplx64 *z_out, const cplx64 *tw,
+                               const StepCoef *coef, const cplx64 *force, cplx64 *z_out, const TwFx *tw,
                                const Dims &d, int tile, cudaStream_t s) {
   return assemble_iz_v<8>(flux, state, (cplx64 *)nullptr, hist, phys, coef, force, z_out, tw, d, tile, s);
 }

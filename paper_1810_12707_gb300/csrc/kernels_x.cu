@@ -18,6 +18,8 @@
 #include "launch_util.cuh"
 #include "tma_util.cuh"
 
+#include <type_traits>
+
 namespace mhd {
 
 namespace {
@@ -67,8 +69,9 @@ constexpr int flux_min_blocks() {
 // so the stages synchronise per group; one block barrier closes the whole transform.
 // Every inverse (DIR = +1) transform here starts from a truncated half spectrum, so its pencil is
 // zero-padded by the 2/3 rule (see pencil_fft).
-template <int N, int DIR, int VPT, typename Ptr, typename C>
-__device__ __forceinline__ void fft_pencils(int np, Ptr ptr, const C *__restrict__ tw) {
+template <int N, int DIR, int VPT, typename Ptr, typename TW>
+__device__ __forceinline__ void fft_pencils(int np, Ptr ptr, const TW *__restrict__ tw) {
+  using C = typename std::remove_pointer<decltype(ptr(0))>::type;
   constexpr int TPP = tpp_for<N, VPT>();
   const int G = blockDim.x / TPP;
   const int g = threadIdx.x / TPP, t = threadIdx.x - g * TPP;
@@ -95,7 +98,7 @@ template <int N, typename C>
 __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restrict__ out,
                                             const PhysDev *__restrict__ phys,
                                             unsigned long long *__restrict__ smax_bits, int K, int blocks_per_inst,
-                                            const C *__restrict__ tw, typename grid_of<C>::type *__restrict__ bgrid,
+                                            const typename tw_of<C>::type *__restrict__ tw, typename grid_of<C>::type *__restrict__ bgrid,
                                             unsigned w, C *sm, double *red) {
   constexpr int KT = (N - 1) / 3;  // the 2/3-rule cut-off, fixed by N
   using R = typename C::value_type;
@@ -297,7 +300,7 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
 template <int N, typename C>
 __global__ void __launch_bounds__((flux_threads<N, C>()), (flux_min_blocks<N, C>()))
     flux_x_kernel(const C *__restrict__ in, C *__restrict__ out, const PhysDev *__restrict__ phys,
-                  unsigned long long *__restrict__ smax_bits, int K, int blocks_per_inst, const C *__restrict__ tw,
+                  unsigned long long *__restrict__ smax_bits, int K, int blocks_per_inst, const typename tw_of<C>::type *__restrict__ tw,
                   typename grid_of<C>::type *__restrict__ bgrid) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
@@ -312,7 +315,7 @@ template <int N, typename C>
 __global__ void __launch_bounds__((flux_threads<N, C>()), (flux_min_blocks<N, C>()))
     flux_x_persistent_kernel(const C *__restrict__ in, C *__restrict__ out, const PhysDev *__restrict__ phys,
                              unsigned long long *__restrict__ smax_bits, int K, int blocks_per_inst,
-                             const C *__restrict__ tw, typename grid_of<C>::type *__restrict__ bgrid, unsigned total,
+                             const typename tw_of<C>::type *__restrict__ tw, typename grid_of<C>::type *__restrict__ bgrid, unsigned total,
                              unsigned *ctr) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
@@ -353,7 +356,7 @@ template <int N, typename C>
 __global__ void __launch_bounds__(kMaxThreads, 1)
     flux_x_pipe_kernel(const C *__restrict__ in, C *__restrict__ out, const PhysDev *__restrict__ phys,
                        unsigned long long *__restrict__ smax_bits, int K, long long total_pairs,
-                       const C *__restrict__ tw, int *err, uint32_t wait_polls) {
+                       const typename tw_of<C>::type *__restrict__ tw, int *err, uint32_t wait_polls) {
   constexpr int KT = (N - 1) / 3;  // the 2/3-rule cut-off, fixed by N
   using R = typename C::value_type;
   extern __shared__ __align__(128) unsigned char smem_pipe[];
@@ -507,12 +510,12 @@ __device__ __forceinline__ void x_load(double v, dfr &r) { r = dfr_from_double(v
 __device__ __forceinline__ double x_store(double v) { return v; }
 __device__ __forceinline__ double x_store(dfr v) { return dfr_to_double(v); }
 
-template <int N, typename C>
+template <int N, typename C, typename TW>
 // Rows from `row_begin` on (a multiple of 2 PAIRS); the real arrays hold rows from `row_begin`
 // with field stride `fstride` (N^3 for whole fields, less for a slab of z-planes).
 __global__ void __launch_bounds__(kMaxThreads) set_x_kernel(const double *__restrict__ rho, const double *__restrict__ u,
                              const double *__restrict__ b, C *__restrict__ out, int K,
-                             const C *__restrict__ tw, size_t row_begin, size_t fstride) {
+                             const TW *__restrict__ tw, size_t row_begin, size_t fstride) {
   using R = typename C::value_type;
   constexpr int KT = (N - 1) / 3;  // the 2/3-rule cut-off, fixed by N
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -563,7 +566,7 @@ __global__ void __launch_bounds__(kMaxThreads) set_x_kernel(const double *__rest
 template <int N, typename C>
 // Rows from `row_begin` on; `out` holds rows from `row_begin` with field stride `fstride`.
 __global__ void __launch_bounds__(kMaxThreads) get_x_kernel(const C *__restrict__ in, double *__restrict__ out, int nf, int K,
-                             const C *__restrict__ tw, size_t row_begin, size_t fstride) {
+                             const typename tw_of<C>::type *__restrict__ tw, size_t row_begin, size_t fstride) {
   constexpr int KT = (N - 1) / 3;  // the 2/3-rule cut-off, fixed by N
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C *sm = reinterpret_cast<C *>(smem_raw);
@@ -611,7 +614,7 @@ __global__ void __launch_bounds__(kMaxThreads) get_x_kernel(const C *__restrict_
 // ------------------------------------------------------------------------------------------
 template <int N>
 __global__ void __launch_bounds__(kMaxThreads) diag_x_kernel(const cplx64 *__restrict__ in, const PhysDev *__restrict__ phys,
-                              double *__restrict__ part, int K, const cplx64 *__restrict__ tw) {
+                              double *__restrict__ part, int K, const TwFx *__restrict__ tw) {
   constexpr int KT = (N - 1) / 3;  // the 2/3-rule cut-off, fixed by N
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx64 *sm = reinterpret_cast<cplx64 *>(smem_raw);
@@ -691,7 +694,7 @@ __global__ void __launch_bounds__(kMaxThreads) diag_x_kernel(const cplx64 *__res
 namespace {
 
 template <int N, typename C>
-cudaError_t flux_n(const C *in, C *out, const PhysDev *phys, unsigned long long *part, const Dims &d, const C *tw,
+cudaError_t flux_n(const C *in, C *out, const PhysDev *phys, unsigned long long *part, const Dims &d, const typename tw_of<C>::type *tw,
                    cudaStream_t s, int *err, typename grid_of<C>::type *bgrid, uint32_t wait_polls, unsigned *ctr) {
   constexpr int PAIRS = pairs_for(N);
   if constexpr (PAIRS == 1 && sizeof(C) == 8) {
@@ -744,9 +747,9 @@ cudaError_t flux_n(const C *in, C *out, const PhysDev *phys, unsigned long long 
   return cudaGetLastError();
 }
 
-template <int N, typename C>
+template <int N, typename C, typename TW>
 cudaError_t set_n(const double *rho, const double *u, const double *b, C *out, const Dims &d,
-                  const C *tw, cudaStream_t s, size_t row_begin, size_t nrows, size_t fstride) {
+                  const TW *tw, cudaStream_t s, size_t row_begin, size_t nrows, size_t fstride) {
   constexpr int PAIRS = pairs_for(N);
   if (row_begin % (2 * PAIRS) || nrows % (2 * PAIRS)) return cudaErrorInvalidValue;
   const int blocks = (int)(nrows / (2 * PAIRS));
@@ -754,15 +757,15 @@ cudaError_t set_n(const double *rho, const double *u, const double *b, C *out, c
   const int threads = threads_for(tpp_for<N, 8>(), 7 * PAIRS);
   const size_t smem = (size_t)7 * PAIRS * pencil_pitch<C>(N) * sizeof(C);
   if (smem > 48 * 1024) {
-    cudaError_t e = ensure_smem<set_x_kernel<N, C>>((int)smem);
+    cudaError_t e = ensure_smem<set_x_kernel<N, C, TW>>((int)smem);
     if (e != cudaSuccess) return e;
   }
-  set_x_kernel<N, C><<<blocks, threads, smem, s>>>(rho, u, b, out, d.k, tw, row_begin, fstride);
+  set_x_kernel<N, C, TW><<<blocks, threads, smem, s>>>(rho, u, b, out, d.k, tw, row_begin, fstride);
   return cudaGetLastError();
 }
 
 template <int N, typename C>
-cudaError_t get_n(const C *in, double *out, int nf, const Dims &d, const C *tw, cudaStream_t s,
+cudaError_t get_n(const C *in, double *out, int nf, const Dims &d, const typename tw_of<C>::type *tw, cudaStream_t s,
                   size_t row_begin, size_t nrows, size_t fstride) {
   constexpr int PAIRS = pairs_for(N);
   if (row_begin % (2 * PAIRS) || nrows % (2 * PAIRS)) return cudaErrorInvalidValue;
@@ -780,7 +783,7 @@ cudaError_t get_n(const C *in, double *out, int nf, const Dims &d, const C *tw, 
 
 template <int N>
 cudaError_t diag_n(const cplx64 *in, const PhysDev *phys, double *part, const Dims &d,
-                   const cplx64 *tw, cudaStream_t s) {
+                   const TwFx *tw, cudaStream_t s) {
   constexpr int PAIRS = pairs_for(N);
   const int blocks = N * N / (2 * PAIRS);
   const int threads = threads_for(tpp_for<N, 8>(), 7 * PAIRS);
@@ -811,7 +814,7 @@ int flux_x_blocks_per_instance(int n) { return n * n / (2 * pairs_for(n)); }
 int diag_x_blocks(int n) { return n * n / (2 * pairs_for(n)); }
 
 cudaError_t launch_flux_x(const cplx64 *in, cplx64 *out, const PhysDev *phys, unsigned long long *smax_bits,
-                          const Dims &d, const cplx64 *tw, cudaStream_t s, int *err, double *bgrid,
+                          const Dims &d, const TwFx *tw, cudaStream_t s, int *err, double *bgrid,
                           uint32_t wait_polls, unsigned *ctr) {
   MHD_DISPATCH_N(d.n, (flux_n<N>(in, out, phys, smax_bits, d, tw, s, err, bgrid, wait_polls, ctr)));
 }
@@ -828,6 +831,17 @@ cudaError_t launch_flux_x(const cdf *in, cdf *out, const PhysDev *phys, unsigned
 }
 
 cudaError_t launch_set_x(const double *rho, const double *u, const double *b, cplx64 *out,
+                         const Dims &d, const TwFx *tw, cudaStream_t s) {
+  const size_t nn = (size_t)d.n * d.n;
+  MHD_DISPATCH_N(d.n, (set_n<N>(rho, u, b, out, d, tw, s, 0, nn, nn * d.n)));
+}
+
+cudaError_t launch_set_x_rows(const double *rho, const double *u, const double *b, cplx64 *out, const Dims &d,
+                              const TwFx *tw, cudaStream_t s, size_t row_begin, size_t nrows, size_t fstride) {
+  MHD_DISPATCH_N(d.n, (set_n<N>(rho, u, b, out, d, tw, s, row_begin, nrows, fstride)));
+}
+
+cudaError_t launch_set_x(const double *rho, const double *u, const double *b, cplx64 *out,
                          const Dims &d, const cplx64 *tw, cudaStream_t s) {
   const size_t nn = (size_t)d.n * d.n;
   MHD_DISPATCH_N(d.n, (set_n<N>(rho, u, b, out, d, tw, s, 0, nn, nn * d.n)));
@@ -839,12 +853,12 @@ cudaError_t launch_set_x_rows(const double *rho, const double *u, const double *
 }
 
 cudaError_t launch_get_x(const cplx64 *in, double *out, int nfields, const Dims &d,
-                         const cplx64 *tw, cudaStream_t s) {
+                         const TwFx *tw, cudaStream_t s) {
   const size_t nn = (size_t)d.n * d.n;
   MHD_DISPATCH_N(d.n, (get_n<N>(in, out, nfields, d, tw, s, 0, nn, nn * d.n)));
 }
 
-cudaError_t launch_get_x_rows(const cplx64 *in, double *out, int nfields, const Dims &d, const cplx64 *tw,
+cudaError_t launch_get_x_rows(const cplx64 *in, double *out, int nfields, const Dims &d, const TwFx *tw,
                               cudaStream_t s, size_t row_begin, size_t nrows, size_t fstride) {
   MHD_DISPATCH_N(d.n, (get_n<N>(in, out, nfields, d, tw, s, row_begin, nrows, fstride)));
 }
@@ -860,7 +874,7 @@ cudaError_t launch_get_x_rows(const cdf *in, double *out, int nfields, const Dim
 }
 
 cudaError_t launch_diag_x(const cplx64 *in, const PhysDev *phys, double *part, const Dims &d,
-                          const cplx64 *tw, cudaStream_t s) {
+                          const TwFx *tw, cudaStream_t s) {
   MHD_DISPATCH_N(d.n, (diag_n<N>(in, phys, part, d, tw, s)));
 }
 

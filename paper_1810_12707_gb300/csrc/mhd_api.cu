@@ -38,7 +38,9 @@ struct mhd_ctx {
   std::vector<char> is_set;
   mhd::PhysDev *phys = nullptr;
   int precision = MHD_FP64;
-  cplx64 *S = nullptr, *H = nullptr, *W1 = nullptr, *W2 = nullptr, *tw = nullptr;
+  cplx64 *S = nullptr, *H = nullptr, *W1 = nullptr, *W2 = nullptr;
+  mhd::TwFx *tw = nullptr;
+  cplx64 *tw_ieee = nullptr;  // mixed mode: the table of the set's IEEE FP64 transforms
   cplx32 *tw32 = nullptr;
   cdf *twdf = nullptr;    // double-float mode: W_N^m as double-float values
   cplx64 *S64 = nullptr;  // mixed and double-float modes: FP64 copy of one instance's state for set/get/diagnostics
@@ -194,6 +196,7 @@ Sizes sizes_for(const mhd::Dims &d, int precision) {
 size_t footprint(const mhd::Dims &d, int precision) {
   const Sizes s = sizes_for(d, precision);
   return (2 * s.S + s.W1 + s.W2) * sizeof(cplx64) + mhd::fp64_twiddle_size(d.n) + d.n * sizeof(cplx32) +
+         (precision == MHD_FP32_MIXED ? mhd::ieee_twiddle_size(d.n) : 0) +
          (precision == MHD_FP64_DF ? d.n * sizeof(cdf) : 0) +
          s.part * sizeof(double) +
          (precision == MHD_FP64 ? 0 : 7 * d.spec * sizeof(cplx64)) +
@@ -385,7 +388,9 @@ mhd_status mhd_init(const mhd_params *p, const mhd_phys *phys, mhd_ctx **out) {
   ok = ok && (c->H = (cplx64 *)dalloc(c, s.S * sizeof(cplx64))) != nullptr;
   ok = ok && (c->W1 = (cplx64 *)dalloc(c, s.W1 * sizeof(cplx64))) != nullptr;
   ok = ok && (c->W2 = (cplx64 *)dalloc(c, s.W2 * sizeof(cplx64))) != nullptr;
-  ok = ok && (c->tw = (cplx64 *)dalloc(c, mhd::fp64_twiddle_size(c->d.n))) != nullptr;
+  ok = ok && (c->tw = (mhd::TwFx *)dalloc(c, mhd::fp64_twiddle_size(c->d.n))) != nullptr;
+  if (c->precision == MHD_FP32_MIXED)
+    ok = ok && (c->tw_ieee = (cplx64 *)dalloc(c, mhd::ieee_twiddle_size(c->d.n))) != nullptr;
   ok = ok && (c->tw32 = (cplx32 *)dalloc(c, (size_t)c->d.n * sizeof(cplx32))) != nullptr;
   if (c->precision != MHD_FP64) ok = ok && (c->S64 = (cplx64 *)dalloc(c, 7 * c->d.spec * sizeof(cplx64))) != nullptr;
   if (c->precision == MHD_FP64_DF) ok = ok && (c->twdf = (cdf *)dalloc(c, (size_t)c->d.n * sizeof(cdf))) != nullptr;
@@ -408,13 +413,16 @@ mhd_status mhd_init(const mhd_params *p, const mhd_phys *phys, mhd_ctx **out) {
   std::vector<mhd::PhysDev> pd(p->batch);
   for (int i = 0; i < p->batch; ++i) pd[i] = mhd::make_phys(phys[i].nu, phys[i].eta, phys[i].cs);
   const std::vector<cplx64> w = mhd::twiddle_table(c->d.n);
-  const std::vector<unsigned char> w64 = mhd::fp64_twiddle_bytes(c->d.n);
+  const std::vector<mhd::TwFx> w64 = mhd::fp64_twiddles(c->d.n);
+  const std::vector<unsigned char> wie = mhd::ieee_twiddle_bytes(c->d.n);
   std::vector<cplx32> w32(w.size());
   for (size_t i = 0; i < w.size(); ++i) w32[i] = cplx32{(float)w[i].re, (float)w[i].im};
   std::vector<cdf> wdf(w.size());
   for (size_t i = 0; i < w.size(); ++i) wdf[i] = cdf{mhd::dfr_const(w[i].re), mhd::dfr_const(w[i].im)};
   cudaError_t e = cudaMemcpyAsync(c->phys, pd.data(), pd.size() * sizeof(mhd::PhysDev), cudaMemcpyHostToDevice, c->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(c->tw, w64.data(), w64.size(), cudaMemcpyHostToDevice, c->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(c->tw, w64.data(), w64.size() * sizeof(mhd::TwFx), cudaMemcpyHostToDevice, c->stream);
+  if (e == cudaSuccess && c->tw_ieee)
+    e = cudaMemcpyAsync(c->tw_ieee, wie.data(), wie.size(), cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->tw32, w32.data(), w32.size() * sizeof(cplx32), cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess && c->twdf)
     e = cudaMemcpyAsync(c->twdf, wdf.data(), wdf.size() * sizeof(cdf), cudaMemcpyHostToDevice, c->stream);
@@ -486,8 +494,8 @@ mhd_status ensure_copy_stream(mhd_ctx *c) {
 // queueing anything when no staging plan fits (the caller then takes the unpipelined path).
 // C = cplx64: FP64 transforms into FP64 spectra; C = cdf: double-float transforms into the
 // double-float state (the values are split at the x pass).
-template <typename C>
-mhd_status set_state_host(mhd_ctx *c, const double *rho, const double *u, const double *b, C *Si, const C *tw) {
+template <typename C, typename TW>
+mhd_status set_state_host(mhd_ctx *c, const double *rho, const double *u, const double *b, C *Si, const TW *tw) {
   SlabPlan pl;
   if (!slab_plan(c, &pl)) return MHD_EINVAL;
   mhd_status st = ensure_copy_stream(c);
@@ -579,7 +587,7 @@ mhd_status async_staging(mhd_ctx *c, Staging *sg) {
 // return once the copies have landed; otherwise the copies are still in flight on sg.cs when it
 // returns (ev_out_done marks their end).
 template <typename C>
-mhd_status get_state_staged(mhd_ctx *c, const C *src, const C *tw, double *rho, double *m, double *b,
+mhd_status get_state_staged(mhd_ctx *c, const C *src, const typename mhd::tw_of<C>::type *tw, double *rho, double *m, double *b,
                             const Staging &sg, bool wait) {
   const mhd::Dims &d = c->d;
   const mhd::Dims d1 = one(c);
@@ -628,7 +636,7 @@ mhd_status get_state_staged(mhd_ctx *c, const C *src, const C *tw, double *rho, 
 // Truncated spectra `src` of one instance -> host rho, m, B through the staging slots in W1.
 // MHD_EINVAL (nothing queued) when no staging plan fits.
 template <typename C>
-mhd_status get_state_host(mhd_ctx *c, const C *src, const C *tw, double *rho, double *m, double *b) {
+mhd_status get_state_host(mhd_ctx *c, const C *src, const typename mhd::tw_of<C>::type *tw, double *rho, double *m, double *b) {
   SlabPlan pl;
   if (!slab_plan(c, &pl)) return MHD_EINVAL;
   mhd_status st = ensure_copy_stream(c);
@@ -676,7 +684,8 @@ mhd_status mhd_set_state(mhd_ctx *c, int32_t inst, const double *rho, const doub
     } else if (st) {
       return st;
     }
-  } else if (!on_device && (st = set_state_host(c, rho, u, b, Si, c->tw)) != MHD_EINVAL) {
+  } else if (!on_device && (st = fp64 ? set_state_host(c, rho, u, b, Si, c->tw)
+                                      : set_state_host(c, rho, u, b, Si, c->tw_ieee)) != MHD_EINVAL) {
     if (st) return st;
   } else {
     const double *r = rho, *uu = u, *bb = b;
@@ -689,9 +698,15 @@ mhd_status mhd_set_state(mhd_ctx *c, int32_t inst, const double *rho, const doub
       uu = real + n3;
       bb = real + 4 * n3;
     }
-    CK(mhd::launch_set_x(r, uu, bb, c->W2, one(c), c->tw, c->stream));
-    CK(mhd::launch_col_forward(c->W2, c->W1, d.n, 7 * d.n, d.nx, 1.0, c->tw, c->stream));
-    CK(mhd::launch_col_forward(c->W1, Si, d.n, 7, d.nk * d.nx, 1.0 / ((double)n3), c->tw, c->stream));
+    auto transform = [&](const auto *tw) {
+      cudaError_t e = mhd::launch_set_x(r, uu, bb, c->W2, one(c), tw, c->stream);
+      if (e == cudaSuccess) e = mhd::launch_col_forward(c->W2, c->W1, d.n, 7 * d.n, d.nx, 1.0, tw, c->stream);
+      if (e == cudaSuccess)
+        e = mhd::launch_col_forward(c->W1, Si, d.n, 7, d.nk * d.nx, 1.0 / ((double)n3), tw, c->stream);
+      return e;
+    };
+    if (fp64) CK(transform(c->tw));
+    else CK(transform(c->tw_ieee));
   }
   if (fp64) {
     CK(cudaMemsetAsync(c->H + (size_t)inst * 7 * d.spec, 0, 7 * d.spec * sizeof(cplx64), c->stream));
@@ -805,7 +820,7 @@ static cudaError_t prof_end(mhd_ctx *c, bool on) {
 // skipped and the inverse y pass reads it.
 template <typename CF, typename CS>
 static mhd_status flux_spectra_t(mhd_ctx *c, const mhd::Dims &d, int inst0, const CS *S, const mhd::PhysDev *phys,
-                                 mhd::TimeState *ts, mhd::StepCoef *coef, bool advance, const CF *tw,
+                                 mhd::TimeState *ts, mhd::StepCoef *coef, bool advance, const typename mhd::tw_of<CF>::type *tw,
                                  typename mhd::grid_of<CF>::type *bgrid, const CF *z_in = nullptr) {
   const int b = d.batch;
   const bool prof = advance && c->profiling;

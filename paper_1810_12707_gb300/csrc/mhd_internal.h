@@ -34,6 +34,22 @@ struct alignas(2 * sizeof(R)) cplx {
 using cplx64 = cplx<double>;
 using cplx32 = cplx<float>;
 
+// One fixed-point twiddle W of the FP64 transforms (fixed64.cuh): -Re W and Im W times 2^62 (2^(62-s)
+// in copy s of a table), each as h 2^32 + l with l in [-2^31, 2^31).
+struct alignas(16) TwFx {
+  int32_t ch, cl, sh, sl;
+};
+constexpr int kFxShifts = 4;
+// Type of the twiddles a pass over values of type C reads.
+template <typename C>
+struct tw_of {
+  using type = C;
+};
+template <>
+struct tw_of<cplx64> {
+  using type = TwFx;
+};
+
 // Per-instance time-stepping state, device resident.
 struct TimeState {
   double t;            // simulated time
@@ -109,27 +125,31 @@ inline Dims make_dims(int n, int batch) {
 }
 
 // ---- launchers (each returns the launch status; all work goes on `s`) ----
-// The FFT passes exist in two precisions: FP64 throughout, and FP32 arithmetic and storage
-// (the first inverse pass reads the FP64 state and writes FP32).  The transform arithmetic runs
-// in the precision of the output; `tw` is the table W_N^m = exp(-2 pi i m / N), m < N, rounded to
-// that precision.
+// The FFT passes exist in FP64 (data in FP64, each pencil transformed in 64-bit fixed point, `tw`
+// a fp64_twiddles table), in double-float, and in FP32 arithmetic and storage, where `tw` is the
+// table W_N^m = exp(-2 pi i m / N), m < N, rounded to that precision.  The transform arithmetic
+// runs in the precision of the output.
 
 // Column FFTs along the middle axis of [nslab][L][C]: inverse (sign +1) expands L from the
 // NK kept indices to N; forward (sign -1) keeps only the NK kept outputs and multiplies by
 // `scale`.
 // `tile` > 0 forces the number of columns per block (else the library's choice).
 // Host twiddle tables (twiddles.cu).  twiddle_table: W_N^m = exp(-2 pi i m/N), m < N.
-// fp64_twiddle_bytes: the table every FP64 transform reads, fp64_twiddle_size(n) bytes: the
-// classic table, then N pairs (c, t), then N bytes q with W_N^m = i^q c (1 + i t), |t| <= 1.
+// fp64_twiddles: the table the FP64 transforms read, kFxShifts copies of W_N^m in 62-bit fixed
+// point, copy s scaled by 2^-s.  ieee_twiddle_bytes: the table of the IEEE FP64 transforms (the
+// mixed mode's set), ieee_twiddle_size(n) bytes: the classic table, then N pairs (c, t), then N
+// bytes q with W_N^m = i^q c (1 + i t), |t| <= 1.
 std::vector<cplx64> twiddle_table(int n);
-std::vector<unsigned char> fp64_twiddle_bytes(int n);
-constexpr size_t fp64_twiddle_size(int n) { return (size_t)n * (2 * sizeof(cplx64) + 1); }
+std::vector<TwFx> fp64_twiddles(int n);
+constexpr size_t fp64_twiddle_size(int n) { return (size_t)kFxShifts * n * sizeof(TwFx); }
+std::vector<unsigned char> ieee_twiddle_bytes(int n);
+constexpr size_t ieee_twiddle_size(int n) { return (size_t)n * (2 * sizeof(cplx64) + 1); }
 
 // `ctr` (nullable): two zeroed unsigned words of device memory owned by the caller; when given,
 // the pass runs as a persistent kernel (one grid of resident blocks taking tiles from ctr[0]) and
 // leaves the words zeroed again.  Results are the same bits either way.
 cudaError_t launch_col_inverse(const cplx64 *in, cplx64 *out, int n, int nslab, int cols,
-                               const cplx64 *tw, cudaStream_t s, int tile = 0, int vpt = 0, unsigned *ctr = nullptr);
+                               const TwFx *tw, cudaStream_t s, int tile = 0, int vpt = 0, unsigned *ctr = nullptr);
 cudaError_t launch_col_inverse(const cplx64 *in, cplx32 *out, int n, int nslab, int cols,
                                const cplx32 *tw, cudaStream_t s, int tile = 0);
 // vpt (FP32 passes): values per thread of the transform, 8 (radix 8) or 16 (radix 16); 0 = the
@@ -140,8 +160,12 @@ cudaError_t launch_col_inverse(const cplx32 *in, cplx32 *out, int n, int nslab, 
 // dir +1 inverse, -1 forward; fp64 the transform type; mixed_in an FP64 input to an FP32 inverse.
 int col_max_tile(int n, int dir, bool fp64, bool mixed_in = false, int vpt = 8);
 cudaError_t launch_col_forward(const cplx64 *in, cplx64 *out, int n, int nslab, int cols,
-                               double scale, const cplx64 *tw, cudaStream_t s, int tile = 0, int vpt = 0,
+                               double scale, const TwFx *tw, cudaStream_t s, int tile = 0, int vpt = 0,
                                unsigned *ctr = nullptr);
+// The same, and the forward x pass of launch_set_x and launch_set_x_rows below, in IEEE FP64
+// arithmetic (an ieee_twiddle_bytes table): the mixed mode's set.
+cudaError_t launch_col_forward(const cplx64 *in, cplx64 *out, int n, int nslab, int cols,
+                               double scale, const cplx64 *tw, cudaStream_t s);
 cudaError_t launch_col_forward(const cplx32 *in, cplx32 *out, int n, int nslab, int cols,
                                double scale, const cplx32 *tw, cudaStream_t s, int tile = 0, int vpt = 0,
                                unsigned *ctr = nullptr);
@@ -165,7 +189,7 @@ constexpr uint32_t kWaitPolls = 1u << 22;
 // `ctr` (nullable, not with the pipelined variant): two zeroed unsigned words; the pass then runs
 // as a persistent kernel taking row-pair blocks from ctr[0] (same results).
 cudaError_t launch_flux_x(const cplx64 *in, cplx64 *out, const PhysDev *phys, unsigned long long *smax_bits,
-                          const Dims &d, const cplx64 *tw, cudaStream_t s, int *err = nullptr,
+                          const Dims &d, const TwFx *tw, cudaStream_t s, int *err = nullptr,
                           double *bgrid = nullptr, uint32_t wait_polls = kWaitPolls, unsigned *ctr = nullptr);
 cudaError_t launch_flux_x(const cplx32 *in, cplx32 *out, const PhysDev *phys, unsigned long long *smax_bits,
                           const Dims &d, const cplx32 *tw, cudaStream_t s, int *err = nullptr,
@@ -180,18 +204,22 @@ int flux_x_blocks_per_instance(int n);
 // Forward real transform along x of 7 real fields given as rho, u (3), B (3) on the grid, with
 // the momentum m = rho u formed first: [7][N^3] real of ONE instance -> [7][z][y][kx <= K].
 cudaError_t launch_set_x(const double *rho, const double *u, const double *b, cplx64 *out,
+                         const Dims &d, const TwFx *tw, cudaStream_t s);
+cudaError_t launch_set_x(const double *rho, const double *u, const double *b, cplx64 *out,
                          const Dims &d, const cplx64 *tw, cudaStream_t s);
 // Inverse real transform along x of `nfields` fields of one instance: [f][z][y][kx <= K] ->
 // real [f][N^3].
 cudaError_t launch_get_x(const cplx64 *in, double *out, int nfields, const Dims &d,
-                         const cplx64 *tw, cudaStream_t s);
+                         const TwFx *tw, cudaStream_t s);
 // The same two x passes over rows [row_begin, row_begin + nrows) only (a slab of z-planes: row =
 // z N + y), with the real arrays holding just those rows, field stride `fstride` doubles.
 // row_begin and nrows must be multiples of the kernels' row-pair block (N >= 16: a multiple of N
 // suffices).
 cudaError_t launch_set_x_rows(const double *rho, const double *u, const double *b, cplx64 *out, const Dims &d,
+                              const TwFx *tw, cudaStream_t s, size_t row_begin, size_t nrows, size_t fstride);
+cudaError_t launch_set_x_rows(const double *rho, const double *u, const double *b, cplx64 *out, const Dims &d,
                               const cplx64 *tw, cudaStream_t s, size_t row_begin, size_t nrows, size_t fstride);
-cudaError_t launch_get_x_rows(const cplx64 *in, double *out, int nfields, const Dims &d, const cplx64 *tw,
+cudaError_t launch_get_x_rows(const cplx64 *in, double *out, int nfields, const Dims &d, const TwFx *tw,
                               cudaStream_t s, size_t row_begin, size_t nrows, size_t fstride);
 // The same in double-float: FP64 values (and the FP64 product rho u) split into double-float pairs
 // on the way in, double-float values summed into FP64 on the way out; transforms in double-float.
@@ -202,7 +230,7 @@ cudaError_t launch_get_x_rows(const cdf *in, double *out, int nfields, const Dim
 // Inverse x pass of the 7 state fields of one instance with per-block partial sums of the grid
 // diagnostics: part[block][8] = (sum ke, me, eint, u.B, |u|, |B|, max s, unused).
 cudaError_t launch_diag_x(const cplx64 *in, const PhysDev *phys, double *part, const Dims &d,
-                          const cplx64 *tw, cudaStream_t s);
+                          const TwFx *tw, cudaStream_t s);
 int diag_x_blocks(int n);
 
 // dt of every instance from its CFL maximum (or the fixed dt), the AB2 coefficients of this
@@ -262,7 +290,7 @@ cudaError_t launch_combine_state(const cdf *in, cplx64 *out, size_t count, cudaS
 // `tile`: columns per block (0 picks).  Mixed mode: s_hi / s_lo the state's parts, `vpt` the
 // inverse z pass's radix option.
 cudaError_t launch_assemble_iz(const cplx64 *flux, cplx64 *state, cplx64 *hist, const PhysDev *phys,
-                               const StepCoef *coef, const cplx64 *force, cplx64 *z_out, const cplx64 *tw,
+                               const StepCoef *coef, const cplx64 *force, cplx64 *z_out, const TwFx *tw,
                                const Dims &d, int tile, cudaStream_t s);
 cudaError_t launch_assemble_iz(const cdf *flux, cdf *state, cdf *hist, const PhysDev *phys, const StepCoef *coef,
                                const cdf *force, cdf *z_out, const cdf *tw, const Dims &d, int tile, cudaStream_t s);
@@ -278,7 +306,7 @@ cudaError_t launch_assemble_iz(const cplx32 *flux, cplx32 *s_hi, cplx32 *s_lo, c
 // dh = i k_x u_hat_x and gh = i k . B_hat on every kept mode.  launch_moments: part[b][2] =
 // (sum v^2, sum v^3) of a fixed share of v; launch_absmax: part[b] = max |v| of a fixed share.
 int num_shells(int k);
-cudaError_t launch_velocity_x(const cplx64 *in, cplx64 *out, const Dims &d, const cplx64 *tw, cudaStream_t s);
+cudaError_t launch_velocity_x(const cplx64 *in, cplx64 *out, const Dims &d, const TwFx *tw, cudaStream_t s);
 cudaError_t launch_shells(const cplx64 *uh, const cplx64 *bh, cplx64 *dh, cplx64 *gh, double *out, const Dims &d,
                           cudaStream_t s);
 cudaError_t launch_moments(const double *v, size_t n, double *part, int blocks, cudaStream_t s);

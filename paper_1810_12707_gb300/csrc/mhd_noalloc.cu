@@ -96,9 +96,9 @@ cudaError_t setup_device(unsigned char **base) {
     e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
     if (e != cudaSuccess) return e;
     unsigned char *b = static_cast<unsigned char *>(p);
-    const std::vector<unsigned char> t16 = mhd::fp64_twiddle_bytes(16), t32 = mhd::fp64_twiddle_bytes(32);
-    e = cudaMemcpy(b + kOffTw16, t16.data(), t16.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(b + kOffTw32, t32.data(), t32.size(), cudaMemcpyHostToDevice);
+    const std::vector<mhd::TwFx> t16 = mhd::fp64_twiddles(16), t32 = mhd::fp64_twiddles(32);
+    e = cudaMemcpy(b + kOffTw16, t16.data(), mhd::fp64_twiddle_size(16), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(b + kOffTw32, t32.data(), mhd::fp64_twiddle_size(32), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return e;
     g_base[dev] = b;
@@ -136,7 +136,7 @@ extern "C" MHD_API mhd_status mhd_rhs_noalloc(int32_t n, const mhd_phys *phys, c
   cplx64 *W1 = reinterpret_cast<cplx64 *>(base + kOffW1);
   cplx64 *W2 = reinterpret_cast<cplx64 *>(base + kOffW2);
   double *part = reinterpret_cast<double *>(base + kOffPart);
-  const cplx64 *tw = reinterpret_cast<const cplx64 *>(base + (n == 16 ? kOffTw16 : kOffTw32));
+  const mhd::TwFx *tw = reinterpret_cast<const mhd::TwFx *>(base + (n == 16 ? kOffTw16 : kOffTw32));
   mhd::PhysDev *pd = reinterpret_cast<mhd::PhysDev *>(base + kOffPhys);
   set_phys_kernel<<<1, 1, 0, s>>>(pd, phys->nu, phys->eta, phys->cs);
   NA_CK(cudaGetLastError());

@@ -4,6 +4,7 @@
 
 #include <vector>
 
+#include "fixed64.cuh"
 #include "mhd_internal.h"
 
 namespace mhd {
@@ -43,12 +44,41 @@ std::vector<cplx64> twiddle_table(int n) {
   return w;
 }
 
-// The FP64 table: the classic table above, then for every m the pair (c, t) and the byte q with
-// W_N^m = i^q c (1 + i t), |t| <= 1.  With q' = the nearest integer to 4m/N, W_N^m =
+// The FP64 table (TwFx): -Re W and Im W times 2^(62 - s) for the copies s = 0..3, rounded to
+// integers and split into h 2^32 + l with l in [-2^31, 2^31).
+std::vector<TwFx> fp64_twiddles(int n) {
+  std::vector<TwFx> t((size_t)kFxShifts * n);
+  auto split = [](int64_t v, int32_t *h, int32_t *l) {
+    *l = (int32_t)(uint32_t)(uint64_t)v;
+    *h = (int32_t)((v - *l) >> 32);
+  };
+  for (int m = 0; m < n; ++m) {
+    // quarter q and the angle's remainder, reflected into the first octant
+    const int q4 = n / 4, quad = m / q4, r = m % q4;
+    const bool flip = r > n / 8;
+    const int a = flip ? q4 - r : r;
+    const long double c0 = a ? cosl(kTwoPi * a / n) : 1.0L, s0 = a ? sinl(kTwoPi * a / n) : 0.0L;
+    long double c = flip ? s0 : c0, s = flip ? c0 : s0;  // cos, sin of 2 pi r / n
+    for (int k = 0; k < quad; ++k) {
+      const long double u = c;
+      c = -s;
+      s = u;
+    }
+    for (int k = 0; k < kFxShifts; ++k) {
+      TwFx &w = t[(size_t)k * n + m];
+      split(llrintl(ldexpl(-c, 62 - k)), &w.ch, &w.cl);
+      split(llrintl(ldexpl(-s, 62 - k)), &w.sh, &w.sl);  // W = exp(-i x): Im W = -sin x
+    }
+  }
+  return t;
+}
+
+// The table of the IEEE FP64 transforms: the classic table above, then for every m the pair (c, t)
+// and the byte q with W_N^m = i^q c (1 + i t), |t| <= 1.  With q' = the nearest integer to 4m/N, W_N^m =
 // i^(-q') exp(2 pi i d / N), d = q' N/4 - m in [-N/8, N/8]: c = cos(2 pi d/N), t = tan(2 pi d/N).
-std::vector<unsigned char> fp64_twiddle_bytes(int n) {
+std::vector<unsigned char> ieee_twiddle_bytes(int n) {
   const std::vector<cplx64> w = twiddle_table(n);
-  std::vector<unsigned char> out(fp64_twiddle_size(n));
+  std::vector<unsigned char> out(ieee_twiddle_size(n));
   memcpy(out.data(), w.data(), (size_t)n * sizeof(cplx64));
   double *ct = reinterpret_cast<double *>(out.data() + (size_t)n * sizeof(cplx64));
   unsigned char *q = out.data() + (size_t)n * 2 * sizeof(cplx64);
