@@ -235,30 +235,26 @@ __device__ __forceinline__ cdf tw_load(const cdf *p) {
                : "l"(p));
   return v;
 }
-// The same from a generic address (a twiddle table a block has staged in shared memory).
-__device__ __forceinline__ cdf tw_load_generic(const cdf *p) {
+// The same from a table that a block has staged in shared memory: element i.
+__device__ __forceinline__ cdf tw_load_shared(const cdf *table, unsigned i) {
   cdf v;
-  asm volatile("ld.v4.f32 {%0, %1, %2, %3}, [%4];"
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
                : "=f"(v.re.hi), "=f"(v.re.lo), "=f"(v.im.hi), "=f"(v.im.lo)
-               : "l"(p));
+               : "r"((unsigned)__cvta_generic_to_shared(table) + i * (unsigned)sizeof(cdf)));
   return v;
 }
-__device__ __forceinline__ cplx64 tw_load(const cplx64 *p) {
-  cplx64 v;
-  asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.re), "=d"(v.im) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ TwFx tw_load(const TwFx *p) {
-  TwFx v;
-  asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v.ch), "=r"(v.cl), "=r"(v.sh), "=r"(v.sl)
-               : "l"(p));
-  return v;
-}
-__device__ __forceinline__ cplx32 tw_load(const cplx32 *p) {
-  cplx32 v;
-  asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.re), "=f"(v.im) : "l"(p));
-  return v;
+// table + kt r.  N >= 512: as one multiply-add (512^3 flux pass, FP32 5.35 -> 5.05 ms, double-float
+// 17.17 -> 17.07); below, left to the compiler (256^3 flux pass 0.559 -> 0.547 and 1.948 -> 1.912 ms,
+// the other way round).
+template <int N, typename W>
+__device__ __forceinline__ const W *tw_at(const W *table, unsigned kt, int r) {
+  if constexpr (N >= 512) {
+    const W *p;
+    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(p) : "r"(kt), "r"((unsigned)(r * (int)sizeof(W))), "l"(table));
+    return p;
+  } else {
+    return table + kt * (unsigned)r;
+  }
 }
 
 // The value of x, opaque to the optimiser: index arithmetic derived from it cannot be hoisted out
@@ -275,9 +271,17 @@ __device__ __forceinline__ int launder(int x) {
 // of a wavefront would hit the same banks.  Pencils are `pencil_pitch` apart, an odd number of
 // elements, so that lanes walking across pencils (the column loads) also spread over the banks.
 template <typename C>
-__host__ __device__ constexpr int sm_idx(int e) { return e + e / (int)(128 / sizeof(C)); }
+__host__ __device__ constexpr int sm_pad() { return (int)(128 / sizeof(C)); }
+template <typename C>
+__host__ __device__ constexpr int sm_idx(int e) { return e + e / sm_pad<C>(); }
 template <typename C>
 __host__ __device__ constexpr int pencil_pitch(int n) { return sm_idx<C>(n) | 1; }
+// The same of an unsigned element index (a shift, where the signed division also handles negatives).
+// sm_at(e) + sm_idx(d) = sm_at(e + d) when d is a multiple of sm_pad, or when no carry leaves the low
+// log2(sm_pad) bits of e + d: the stages below address a butterfly's elements at constant offsets
+// from its first one.
+template <typename C>
+__device__ __forceinline__ unsigned sm_at(unsigned e) { return e + e / (unsigned)sm_pad<C>(); }
 
 // ---- barrier of one pencil's thread group ----
 // A pencil is transformed by the TPP = N/VPT consecutive threads of its group and nobody else
@@ -490,7 +494,7 @@ __host__ __device__ constexpr int fft_tpp() { return tpp_for<N, fft_vpt<C>()>();
 // Every thread of the block must call this (it contains group barriers); threads with
 // `active == false` only take part in the barriers.  The caller separates the transform from the
 // preceding writes and the following reads of the pencil with a block barrier.
-// TWG: `tw` may point to shared memory (generic twiddle loads; double-float only).
+// TWG: `tw` points to shared memory (double-float only).
 template <int N, int DIR, int NS, typename C, int VPT, bool ZP, bool TWG = false>
 __device__ __forceinline__ void stockham_stages(C *buf, int t, bool active, const C *__restrict__ tw) {
   if constexpr (NS < N) {
@@ -511,21 +515,25 @@ __device__ __forceinline__ void stockham_stages(C *buf, int t, bool active, cons
                   "inputs 3 and 4 of the first radix-8 stage must lie in the 2/3-rule gap");
     static_assert(!kFirst16 || (6 * (N / 16) > K && 10 * (N / 16) - 1 < N - K),
                   "inputs 6..9 of the first radix-16 stage must lie in the 2/3-rule gap");
+    // reads at constant offsets from the butterfly's first element (see sm_at); the smallest grids'
+    // strides are not multiples of the pad's period
+    constexpr bool kConst = (N / R) % sm_pad<C>() == 0;
     C v[VPT];
     if (active) {
 #pragma unroll
       for (int b = 0; b < NB; ++b) {
-        const int j = t + b * TPP;
-        const int k = j % NS;
+        const unsigned j = (unsigned)(t + b * TPP);
+        const unsigned kt = (j % (unsigned)NS) * (unsigned)TWSTEP;
+        const C *rp = buf + sm_at<C>(j);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           if (kFirst && ZP && (r == 3 || r == 4)) continue;  // zeros, never read
           if (kFirst16 && r >= 6 && r <= 9) continue;
-          C x = buf[sm_idx<C>(j + r * (N / R))];
+          C x = kConst ? rp[sm_idx<C>(r * (N / R))] : buf[sm_at<C>(j + r * (N / R))];
           if (!kFma && NS > 1 && r > 0) {
             C w;
-            if constexpr (TWG) w = tw_load_generic(tw + r * k * TWSTEP);
-            else w = tw_load(tw + r * k * TWSTEP);
+            if constexpr (TWG) w = tw_load_shared(tw, kt * (unsigned)r);
+            else w = tw_load(tw_at<N>(tw, kt, r));
             x = DIR < 0 ? c_mul(x, w) : c_mulc(x, w);
           }
           v[b * R + r] = x;
@@ -536,8 +544,10 @@ __device__ __forceinline__ void stockham_stages(C *buf, int t, bool active, cons
     if (active) {
 #pragma unroll
       for (int b = 0; b < NB; ++b) {
+        const unsigned j = (unsigned)(t + b * TPP);
+        const unsigned k = j % (unsigned)NS;
         if constexpr (kFma) {
-          dft_twiddled_fma<N, R, DIR>(reinterpret_cast<cplx64 *>(v) + b * R, ((t + b * TPP) % NS) * TWSTEP,
+          dft_twiddled_fma<N, R, DIR>(reinterpret_cast<cplx64 *>(v) + b * R, (int)(k * TWSTEP),
                                       reinterpret_cast<const cplx64 *>(tw));
         } else if constexpr (kFirst) {
           dft8_first_fma<DIR, ZP>(v + b * R);
@@ -546,11 +556,9 @@ __device__ __forceinline__ void stockham_stages(C *buf, int t, bool active, cons
         } else {
           dft_small<R, DIR, C>(v + b * R);
         }
-        const int j = t + b * TPP;
-        const int k = j % NS;
-        const int base = (j / NS) * NS * R + k;
+        C *wp = buf + sm_at<C>((j - k) * R + k);
 #pragma unroll
-        for (int r = 0; r < R; ++r) buf[sm_idx<C>(base + r * NS)] = v[b * R + r];
+        for (int r = 0; r < R; ++r) wp[sm_idx<C>(r * NS)] = v[b * R + r];
       }
     }
     group_sync<TPP>();
@@ -562,14 +570,15 @@ __device__ __forceinline__ void stockham_stages(C *buf, int t, bool active, cons
 // The same Stockham stages on a pencil of doubles.  The first stage reads doubles, finds the
 // pencil's common exponent and converts; the pencil is fixed-point complex values between the
 // stages; the last stage writes doubles.  Against the IEEE FP64 stages this replaced (FP64 pipe 92 %
-// busy), ms per pass: 512^3 inverse y 12.4 -> 4.13, forward y 23.8 -> 8.54, flux 65.6 -> 27.0;
-// 256^3 step 14.75 -> 5.38.  The exponent's reduction adds no barrier: a group of
+// busy), ms per pass: 512^3 inverse y 12.4 -> 3.98, forward y 23.8 -> 6.60, flux 65.6 -> 21.1;
+// 256^3 step 14.75 -> 4.97.  The exponent's reduction adds no barrier: a group of
 // more than a warp leaves its warps' parts in shared memory before the barrier that the first
 // stage has between its reads and its writes anyway.  It depends on the group's threads only, so
 // a pencil's results are the same bits in every kernel and at every tile width.
-template <int N, int DIR, int NS>
+// DP: the results' conversion runs on the FP64 pipe; `scale2`: they are scaled by 2^scale2.
+template <int N, int DIR, int NS, bool DP>
 __device__ __forceinline__ void fx_stages(cfx *buf, int t, bool active, const TwFx *__restrict__ tw, const FxScale &sc,
-                                          int left) {
+                                          int left, int scale2) {
   constexpr int R = N / NS >= 8 ? 8 : N / NS;
   constexpr int NB = 8 / R;
   constexpr int TPP = tpp_for<N, 8>();
@@ -581,30 +590,35 @@ __device__ __forceinline__ void fx_stages(cfx *buf, int t, bool active, const Tw
     const TwFx *ts = tw + s * N;
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
-      const int j = t + b * TPP;
-      const int k = j % NS;
-      v[b * R] = fx_shift(buf[sm_idx<cplx64>(j)], s);
+      const unsigned j = (unsigned)(t + b * TPP);
+      const unsigned kt = (j % (unsigned)NS) * (unsigned)TWSTEP;
+      static_assert((N / R) % sm_pad<cplx64>() == 0, "constant read offsets");
+      const cfx *rp = buf + sm_at<cplx64>(j);
+      v[b * R] = fx_shift(rp[0], s);
 #pragma unroll
       for (int r = 1; r < R; ++r)
-        v[b * R + r] = fx_mul<DIR>(buf[sm_idx<cplx64>(j + r * (N / R))], tw_load(ts + r * k * TWSTEP));
+        v[b * R + r] = fx_mul<DIR>(rp[sm_idx<cplx64>(r * (N / R))], tw_load(tw_at<N>(ts, kt, r)));
       fx_dft<R, DIR>(v + b * R);
     }
   }
   group_sync<TPP>();
   if (active) {
-    const uint32_t be = sc.ek + (uint32_t)sc.shift + 1u;
+    const uint32_t be = sc.ek + (uint32_t)(sc.shift + scale2) + 1u;
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
-      const int j = t + b * TPP;
-      const int base = (j / NS) * NS * R + j % NS;
+      const unsigned j = (unsigned)(t + b * TPP);
+      const unsigned k = j % (unsigned)NS;
+      cfx *wp = buf + sm_at<cplx64>((j - k) * R + k);
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const cfx x = v[b * R + r];
-        cfx *p = buf + sm_idx<cplx64>(base + r * NS);
+        cfx *p = wp + sm_idx<cplx64>(r * NS);
         if constexpr (NS * R < N) {
           *p = x;
         } else {
-          cplx64 d = {fx_to_double(x.re, be), fx_to_double(x.im, be)};
+          cplx64 d;
+          if constexpr (DP) d = cplx64{fx_to_double_dp(x.re, be), fx_to_double_dp(x.im, be)};
+          else d = cplx64{fx_to_double(x.re, be), fx_to_double(x.im, be)};
           if (sc.bad) d.re = d.im = fx_double(0x7ff80000u, 0u);
           *reinterpret_cast<cplx64 *>(p) = d;
         }
@@ -612,11 +626,12 @@ __device__ __forceinline__ void fx_stages(cfx *buf, int t, bool active, const Tw
     }
   }
   group_sync<TPP>();
-  if constexpr (NS * R < N) fx_stages<N, DIR, NS * R>(buf, t, active, tw, sc, left - s);
+  if constexpr (NS * R < N) fx_stages<N, DIR, NS * R, DP>(buf, t, active, tw, sc, left - s, scale2);
 }
 
-template <int N, int DIR, bool ZP>
-__device__ __forceinline__ void fx_pencil_fft(cplx64 *buf, int t, bool active, const TwFx *__restrict__ tw) {
+template <int N, int DIR, bool ZP, bool DP = false>
+__device__ __forceinline__ void fx_pencil_fft(cplx64 *buf, int t, bool active, const TwFx *__restrict__ tw,
+                                              int scale2 = 0) {
   constexpr int TPP = tpp_for<N, 8>();
   constexpr int LOG2G = TPP == 128 ? 7 : TPP == 64 ? 6 : TPP == 32 ? 5 : TPP == 16 ? 4 : TPP == 8 ? 3 : TPP == 4 ? 2 : 1;
   constexpr int K = (N - 1) / 3;
@@ -627,7 +642,9 @@ __device__ __forceinline__ void fx_pencil_fft(cplx64 *buf, int t, bool active, c
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
     x[r] = cplx64{0.0, 0.0};
-    if (!(ZP && (r == 3 || r == 4)) && active) x[r] = buf[sm_idx<cplx64>(t + r * TPP)];
+    if (!(ZP && (r == 3 || r == 4)) && active)
+      x[r] = TPP % sm_pad<cplx64>() == 0 ? buf[sm_at<cplx64>((unsigned)t) + sm_idx<cplx64>(r * TPP)]
+                                         : buf[sm_at<cplx64>((unsigned)(t + r * TPP))];
   }
   uint32_t m = 0u;
 #pragma unroll
@@ -681,22 +698,33 @@ __device__ __forceinline__ void fx_pencil_fft(cplx64 *buf, int t, bool active, c
     }
     fx_dft8<DIR, ZP>(v);
 #pragma unroll
-    for (int r = 0; r < 8; ++r) fb[sm_idx<cplx64>(8 * t + r)] = v[r];
+    for (int r = 0; r < 8; ++r) fb[9u * (unsigned)t + r] = v[r];
   }
   group_sync<TPP>();
-  fx_stages<N, DIR, 8>(fb, t, active, tw, sc, sc.shift);
+  fx_stages<N, DIR, 8, DP>(fb, t, active, tw, sc, sc.shift, scale2);
 }
 
 // `t` in [0, N / VPT): the thread's index within its pencil's group.  ZP: the pencil is
 // zero-padded by the 2/3 rule (elements K+1 .. N-K-1 are zero, K = (N-1)/3), as every inverse
-// transform of a truncated spectrum is; the FP64 first stage then skips the inputs it knows are
-// zero (they need not even be written).
-// TW: the twiddle table's type; a TwFx table runs an FP64 pencil in fixed point.
-template <int N, int DIR, typename C, int VPT = fft_vpt<C>(), bool ZP = false, bool TWG = false, typename TW>
-__device__ __forceinline__ void pencil_fft(C *buf, int t, bool active, const TW *__restrict__ tw) {
+// transform of a truncated spectrum is; the first stage then skips the inputs it knows are zero,
+// elements 3N/8 .. 5N/8 - 1, which need not be written (pencil_zero_count, pencil_zero).
+// The zeros that do have to be written into a zero-padded pencil: elements K+1 .. 3N/8 - 1 and
+// 5N/8 .. N-K-1; zero number i of pencil_zero_count is element pencil_zero(i).
+template <int N>
+__host__ __device__ constexpr int pencil_zero_count() { return 2 * (3 * (N / 8) - (N - 1) / 3 - 1) + 1; }
+template <int N>
+__device__ __forceinline__ unsigned pencil_zero(unsigned i) {
+  constexpr unsigned K = (N - 1) / 3, A = 3 * (N / 8) - K - 1;  // N-K - 5N/8 = A + 1
+  return i < A ? K + 1 + i : 5 * (N / 8) + (i - A);
+}
+// TW: the twiddle table's type; a TwFx table runs an FP64 pencil in fixed point, with its results
+// converted on the FP64 pipe if DP and scaled by 2^scale2.
+template <int N, int DIR, typename C, int VPT = fft_vpt<C>(), bool ZP = false, bool TWG = false, bool DP = false,
+          typename TW>
+__device__ __forceinline__ void pencil_fft(C *buf, int t, bool active, const TW *__restrict__ tw, int scale2 = 0) {
   if constexpr (std::is_same<TW, TwFx>::value) {
     static_assert(std::is_same<C, cplx64>::value && VPT == 8, "fixed-point transforms are FP64's, radix 8");
-    fx_pencil_fft<N, DIR, ZP>(buf, t, active, tw);
+    fx_pencil_fft<N, DIR, ZP, DP>(buf, t, active, tw, scale2);
   } else {
     stockham_stages<N, DIR, 1, C, VPT, ZP, TWG>(buf, t, active, tw);
   }

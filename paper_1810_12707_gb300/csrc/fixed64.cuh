@@ -16,7 +16,7 @@
 // where an FP64 butterfly rounds at 2^-53 of its values.  Values more than 2^60 below the largest
 // first-stage sum round to zero; in FP64 they are lost in the same butterflies' rounding errors.
 //
-// A pencil with a NaN or an infinity (or a magnitude above 2^1007) transforms to NaN everywhere;
+// A pencil with a NaN or an infinity (or a magnitude above 2^976) transforms to NaN everywhere;
 // one whose largest magnitude is below 2^-959 transforms to zeros.
 #pragma once
 
@@ -143,9 +143,9 @@ FX_FN FxScale fx_scale(FxPart p, int log2_groups) {
   int sh = ct - ca;
   if (sh > log2_groups) sh = log2_groups;  // T is at most (groups) A
   FxScale s;
-  s.ek = p.m < 64u ? 8191u : p.m + 3u + (uint32_t)ca;  // A < 2^60
+  s.ek = p.m < 64u ? 200u : p.m + 3u + (uint32_t)ca;  // A < 2^60
   s.shift = sh;
-  s.bad = p.m >= 2030u;
+  s.bad = p.m >= 2000u;
   return s;
 }
 
@@ -177,6 +177,17 @@ FX_FN double fx_to_double(int64_t v, uint32_t be) {
                      ((uint64_t)((be - n - 1u) << 20) << 32);
   const uint32_t sign = (uint32_t)(v >> 32) & 0x80000000u;
   return zero ? 0.0 : fx_double((uint32_t)(r >> 32) | sign, (uint32_t)r);
+}
+
+// The same on the FP64 pipe: v = h 2^32 + l read into the significands of 2^84 + (h + 2^31) 2^32
+// and 2^52 + l, whose difference and sum with the offsets' total is v, rounded once (to even).  Two
+// additions of the FP64 pipe and one integer instruction instead of about 20 integer ones: for
+// kernels that leave the FP64 pipe idle (the column passes and the set and get passes).  A result
+// below 2^-1022 is rounded as FP64 rounds it.
+FX_FN double fx_to_double_dp(int64_t v, uint32_t be) {
+  const uint32_t eh = (be + 21u) << 20, el = (be - 11u) << 20;
+  const double h = fx_double(eh, (uint32_t)(v >> 32) ^ 0x80000000u), l = fx_double(el, (uint32_t)v);
+  return (h - fx_double(eh, 0x80100000u)) + l;
 }
 
 // ---- butterflies ----

@@ -25,6 +25,34 @@ constexpr bool tws_staged() { return std::is_same<CC, cdf>::value && N >= 512; }
 template <typename CC, int N>
 constexpr size_t tws_bytes() { return tws_staged<CC, N>() ? (size_t)N * sizeof(CC) : 0; }
 
+// Where a thread's rows l = l0 + i TPP (l0 < TPP) lie in a pencil: kept index l at FFT index l, or
+// l + N - NK above K, or (all rows) FFT index l.  Addresses are at constant offsets from two base
+// pointers where TPP is a multiple of the pad's period; only the row group that straddles K needs
+// a selection.
+template <int N, int TPP, typename CC>
+struct KeptRows {
+  static constexpr int K = (N - 1) / 3, UP = N - (2 * K + 1);
+  static constexpr bool kConst = TPP % sm_pad<CC>() == 0;
+  CC *pen, *lo, *hi;
+  unsigned l0;
+  __device__ __forceinline__ KeptRows(CC *p, unsigned l) : pen(p), l0(l) {
+    lo = p + sm_at<CC>(l);
+    hi = p + sm_at<CC>(l + (unsigned)(UP % sm_pad<CC>())) + sm_idx<CC>(UP - UP % sm_pad<CC>());
+  }
+  template <bool Kept>
+  __device__ __forceinline__ CC *row(int i) const {
+    const int d = i * TPP;
+    if constexpr (!kConst) {
+      const unsigned l = l0 + d;
+      return pen + sm_at<CC>(Kept && l > (unsigned)K ? l + UP : l);
+    } else {
+      if (!Kept || d + TPP - 1 <= K) return lo + sm_idx<CC>(d);
+      if (d > K) return hi + sm_idx<CC>(d);
+      return (l0 + d > (unsigned)K ? hi : lo) + sm_idx<CC>(d);
+    }
+  }
+};
+
 // CI, CO: element types in and out; CC: type of the transform arithmetic (= the output's).
 // A block has TC = 2^tsh columns and TC * N/VPT threads: thread (l0, c) = (tid >> tsh, tid & (TC-1))
 // moves rows l0, l0 + N/VPT, ... of column c, so consecutive threads touch consecutive columns of a
@@ -58,16 +86,17 @@ __device__ __forceinline__ void col_fft_tile(const CI *__restrict__ in, CO *__re
   for (int i = 0; i < NLD; ++i) {
     const int l = l0 + i * TPP;
     v[i] = CC{0, 0};
-    if (col_ok && l < LIN) v[i] = c_cvt<CC>(src[(size_t)l * cols]);
+    if (col_ok && (LIN % TPP == 0 || i + 1 < NLD || l < LIN)) v[i] = c_cvt<CC>(src[(size_t)l * cols]);
   }
+  const KeptRows<N, TPP, CC> at(pen, (unsigned)l0);
 #pragma unroll
   for (int i = 0; i < NLD; ++i) {
-    const int l = l0 + i * TPP;
-    if (l < LIN) pen[sm_idx<CC>(DIR > 0 ? kept_to_fft(l, K, N) : l)] = v[i];
+    if (LIN % TPP == 0 || i + 1 < NLD || l0 + i * TPP < LIN) *at.template row<(DIR > 0)>(i) = v[i];
   }
   if (DIR > 0) {
-    // FFT indices K+1 .. N-K-1 are outside the kept set
-    for (int l = l0; l < N - NK; l += TPP) pen[sm_idx<CC>(K + 1 + l)] = CC{0, 0};
+    // of the FFT indices K+1 .. N-K-1, outside the kept set, those that the transform reads
+    for (unsigned l = l0; l < (unsigned)pencil_zero_count<N>(); l += TPP)
+      pen[sm_at<CC>(pencil_zero<N>(l))] = CC{0, 0};
   }
   // double-float at N >= 512: the twiddle table staged in shared memory behind the pencils
   constexpr bool kTws = tws_staged<CC, N>();
@@ -82,15 +111,28 @@ __device__ __forceinline__ void col_fft_tile(const CI *__restrict__ in, CO *__re
   const int pencil = threadIdx.x / TPP;
   const int t = threadIdx.x - pencil * TPP;
   const bool active = pencil < tc && tile * tc + pencil < cols;
-  pencil_fft<N, DIR, CC, VPT, (DIR > 0), kTws>(sm + (active ? pencil : 0) * P, t, active, twp);  // inverse: zero-padded
+  // fixed-point transforms take `scale`, a power of two there, into their results' exponents
+  constexpr bool kFx = std::is_same<TW, TwFx>::value;
+  int scale2 = 0;
+  if constexpr (kFx && DIR < 0) scale2 = (int)fx_exp(fx_hi(scale)) - 1023;
+  pencil_fft<N, DIR, CC, VPT, (DIR > 0), kTws, kFx>(sm + (active ? pencil : 0) * P, t, active, twp,
+                                                     scale2);  // inverse: zero-padded
   __syncthreads();  // the store loop reads every pencil
 
   if (col_ok) {
     CO *dst = out + slab * (size_t)LOUT * cols + col;
-    for (int l = l0; l < LOUT; l += TPP) {
-      CC v = pen[sm_idx<CC>(DIR > 0 ? l : kept_to_fft(l, K, N))];
-      if (DIR < 0 && scale != (typename scale_of<CC>::type)1) v = c_scale(v, scale);
-      dst[(size_t)l * cols] = c_store(c_cvt<CO>(v));
+    // the double-float inverse passes keep their 64 registers (4 blocks per SM) with a short unroll:
+    // 512^3 inverse y 3.24 ms against 3.52
+    constexpr int kStoreUnroll = std::is_same<CC, cdf>::value && DIR > 0 ? 2 : 16;
+    constexpr int NST = (LOUT + TPP - 1) / TPP;
+#pragma unroll(kStoreUnroll)
+    for (int i = 0; i < NST; ++i) {
+      const int l = l0 + i * TPP;
+      if (LOUT % TPP == 0 || i + 1 < NST || l < LOUT) {
+        CC v = *at.template row<(DIR < 0)>(i);
+        if (!kFx && DIR < 0 && scale != (typename scale_of<CC>::type)1) v = c_scale(v, scale);
+        dst[(size_t)l * cols] = c_store(c_cvt<CO>(v));
+      }
     }
   }
 }
@@ -103,9 +145,10 @@ __global__ void col_fft_kernel(const CI *__restrict__ in, CO *__restrict__ out, 
                                         reinterpret_cast<CC *>(smem_raw));
 }
 
-// Double-float forward passes: the same tile with 4 blocks of 256 threads per SM (64 registers a
-// thread), which measured 8 % faster at 512^3 than the 3 blocks that 72 registers allow (the
-// inverse passes measured slower so and keep col_fft_kernel).
+// FP64 passes and double-float forward passes: the same tile with 4 blocks of 256 threads per SM
+// (64 registers a thread).  Against the 3 blocks that 66 to 74 registers allow: FP64 at 512^3
+// inverse y 4.57 -> 3.97 ms, forward y 7.81 -> 6.60 ms; double-float forward y 8 % faster.  (The
+// double-float inverse passes measured slower so and keep col_fft_kernel.)
 template <int N, int DIR, typename CI, typename CO, typename CC, int VPT, typename TW>
 __global__ void __launch_bounds__(256, 4) col_fft_kernel_b4(const CI *__restrict__ in, CO *__restrict__ out,
                                                            int ntiles, int tsh, int cols,
@@ -119,7 +162,7 @@ __global__ void __launch_bounds__(256, 4) col_fft_kernel_b4(const CI *__restrict
 // The kernel a pass launches.
 template <int N, int DIR, typename CI, typename CO, int VPT, typename TW = typename tw_of<CO>::type>
 constexpr auto col_kernel() {
-  if constexpr (std::is_same<CO, cdf>::value && DIR < 0) return col_fft_kernel_b4<N, DIR, CI, CO, CO, VPT, TW>;
+  if constexpr ((std::is_same<CO, cdf>::value && DIR < 0) || std::is_same<TW, TwFx>::value) return col_fft_kernel_b4<N, DIR, CI, CO, CO, VPT, TW>;
   else return col_fft_kernel<N, DIR, CI, CO, CO, VPT, TW>;
 }
 

@@ -73,10 +73,10 @@ __global__ void __launch_bounds__(kMaxThreads) velocity_x_kernel(const cplx64 *_
       pen[sm_idx<cplx64>(N - k)] = cplx64{x0.re + x1.im, x1.re - x0.im};
     }
   }
-  for (int q = threadIdx.x; q < 4 * PAIRS * (N - 2 * KT - 1); q += nthr) {
-    const int z = q % (N - 2 * KT - 1);
-    const int r = q / (N - 2 * KT - 1);
-    sm[r * P + sm_idx<cplx64>(KT + 1 + z)] = cplx64{0.0, 0.0};
+  constexpr int NZ = pencil_zero_count<N>();
+  for (unsigned q = threadIdx.x; q < (unsigned)(4 * PAIRS * NZ); q += nthr) {
+    const unsigned z = q % NZ, r = q / NZ;
+    sm[r * P + sm_at<cplx64>(pencil_zero<N>(z))] = cplx64{0.0, 0.0};
   }
   __syncthreads();
   fft_pencils<N, +1>(4 * PAIRS, [&](int id) { return sm + id * P; }, tw);

@@ -839,10 +839,11 @@ __global__ void __launch_bounds__(fused_max_threads<N, VPT>(), (fused_max_thread
       for (int f = 0; f < 7; ++f) yn[f * tc * P] = C{0, 0};
     }
   }
-  // FFT indices K+1 .. N-K-1 are outside the kept set
-  for (int it = threadIdx.x; it < 7 * tc * (N - NK); it += nthr) {
-    const int p = it / (N - NK), r = it - p * (N - NK);
-    sm[p * P + sm_idx<C>(K + 1 + r)] = C{0, 0};
+  // of the FFT indices K+1 .. N-K-1, outside the kept set, those that the transform reads
+  constexpr int NZ = pencil_zero_count<N>();
+  for (unsigned it = threadIdx.x; it < (unsigned)(7 * tc * NZ); it += nthr) {
+    const unsigned p = it / NZ, z = it % NZ;
+    sm[p * P + sm_at<C>(pencil_zero<N>(z))] = C{0, 0};
   }
   __syncthreads();
 

@@ -40,10 +40,10 @@ constexpr int threads_for(int tpp, int pencils, int max_threads = kMaxThreads) {
 // Block size of the flux pass.  At N = 256 and 512 several smaller blocks per SM let one block
 // transform while another waits at a barrier (measured on GB300 over 96..384 threads: 128 best at
 // 256^3 in both precisions, 192 at 512^3); below, the pencil count caps the block at 192 threads.
-// The double-float pass at 512^3 takes 256 (two blocks of 128 registers a thread per SM): 4 %
-// faster than 192.
-constexpr int flux_max_threads(int n, bool df = false) {
-  return n == 256 ? 128 : n == 512 ? (df ? 256 : 192) : kMaxThreads;
+// The 16-byte passes at 512^3 take 256 (two blocks of 128 registers a thread per SM): double-float
+// 4 % faster than 192, FP64 27.0 -> 22.8 ms.
+constexpr int flux_max_threads(int n, bool wide = false) {
+  return n == 256 ? 128 : n == 512 ? (wide ? 256 : 192) : kMaxThreads;
 }
 // Values per thread of the flux pass's transforms: FP32 at N <= 256 uses radix 16 (measured
 // faster at 64^3 and 256^3); larger FP32 grids and FP64 use radix 8.
@@ -52,14 +52,14 @@ constexpr int flux_vpt() { return sizeof(C) == 8 && N <= 256 ? 16 : 8; }
 template <int N, typename C>
 constexpr int flux_threads() {
   return threads_for(tpp_for<N, flux_vpt<N, C>()>(), 12 * pairs_for(N),
-                     flux_max_threads(N, std::is_same<C, cdf>::value));
+                     flux_max_threads(N, sizeof(C) == 16));
 }
 // Blocks per SM the register allocation is sized for: about 170 registers a thread in FP64, 85 in
 // FP32 with radix 8 and 128 with radix 16 (its 16 values per thread).
 template <int N, typename C>
 constexpr int flux_min_blocks() {
   const int budget = sizeof(C) == 8 ? (flux_vpt<N, C>() == 16 ? 512 : 768)
-                                    : (N == 512 && std::is_same<C, cdf>::value ? 512 : 384);
+                                    : (N == 512 ? 512 : 384);
   const int b = budget / flux_threads<N, C>();
   return b < 1 ? 1 : b;
 }
@@ -69,8 +69,9 @@ constexpr int flux_min_blocks() {
 // so the stages synchronise per group; one block barrier closes the whole transform.
 // Every inverse (DIR = +1) transform here starts from a truncated half spectrum, so its pencil is
 // zero-padded by the 2/3 rule (see pencil_fft).
-template <int N, int DIR, int VPT, typename Ptr, typename TW>
-__device__ __forceinline__ void fft_pencils(int np, Ptr ptr, const TW *__restrict__ tw) {
+// DP, scale2: see pencil_fft.
+template <int N, int DIR, int VPT, bool DP = false, typename Ptr, typename TW>
+__device__ __forceinline__ void fft_pencils(int np, Ptr ptr, const TW *__restrict__ tw, int scale2 = 0) {
   using C = typename std::remove_pointer<decltype(ptr(0))>::type;
   constexpr int TPP = tpp_for<N, VPT>();
   const int G = blockDim.x / TPP;
@@ -78,7 +79,7 @@ __device__ __forceinline__ void fft_pencils(int np, Ptr ptr, const TW *__restric
   for (int base = 0; base < np; base += G) {
     const int id = base + g;
     const bool active = g < G && id < np;
-    pencil_fft<N, DIR, C, VPT, (DIR > 0)>(ptr(active ? id : 0), t, active, tw);
+    pencil_fft<N, DIR, C, VPT, (DIR > 0), false, DP>(ptr(active ? id : 0), t, active, tw, scale2);
   }
   __syncthreads();  // the callers' next phase reads every pencil
 }
@@ -133,11 +134,11 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
       }
     }
   }
-  for (int q = threadIdx.x; q < 7 * PAIRS * (N - 2 * KT - 1); q += nthr) {
-    const int z = q % (N - 2 * KT - 1);
-    const int r = q / (N - 2 * KT - 1);
-    const int f = r % 7, p = r / 7;
-    sm[(p * 12 + f) * P + sm_idx<C>(KT + 1 + z)] = C{0, 0};
+  constexpr int NZ = pencil_zero_count<N>();
+  for (unsigned q = threadIdx.x; q < (unsigned)(7 * PAIRS * NZ); q += nthr) {
+    const unsigned z = q % NZ, r = q / NZ;
+    const unsigned f = r % 7, p = r / 7;
+    sm[(p * 12 + f) * P + sm_at<C>(pencil_zero<N>(z))] = C{0, 0};
   }
   __syncthreads();
 
@@ -429,9 +430,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
         pen[sm_idx<C>(N - k)] = C{x0.re + x1.im, x1.re - x0.im};
       }
     }
-    for (int q = tx; q < 7 * (N - 2 * KT - 1); q += nthr) {
-      const int z = q % (N - 2 * KT - 1), f = q / (N - 2 * KT - 1);
-      sm[f * P + sm_idx<C>(KT + 1 + z)] = C{0, 0};
+    constexpr int NZ = pencil_zero_count<N>();
+    for (unsigned q = tx; q < (unsigned)(7 * NZ); q += nthr) {
+      const unsigned z = q % NZ, f = q / NZ;
+      sm[f * P + sm_at<C>(pencil_zero<N>(z))] = C{0, 0};
     }
     __syncthreads();
 
@@ -547,7 +549,13 @@ __global__ void __launch_bounds__(kMaxThreads) set_x_kernel(const double *__rest
     }
   }
   __syncthreads();
-  fft_pencils<N, -1, 8>(7 * PAIRS, [&](int id) { return sm + id * P; }, tw);
+  // the split's factor 1/2: in fixed point a step of the results' exponents
+  constexpr bool kFx = std::is_same<TW, TwFx>::value;
+  fft_pencils<N, -1, 8, kFx>(7 * PAIRS, [&](int id) { return sm + id * P; }, tw, kFx ? -1 : 0);
+  const auto half = [](C v) {
+    if constexpr (kFx) return v;
+    else return c_scale(v, (typename scale_of<C>::type)0.5);
+  };
   for (int q = threadIdx.x; q < 7 * PAIRS * NX; q += nthr) {
     const int k = q % NX;
     const int r = q / NX;
@@ -555,8 +563,8 @@ __global__ void __launch_bounds__(kMaxThreads) set_x_kernel(const double *__rest
     const C *pen = sm + (p * 7 + f) * P;
     const C z = pen[sm_idx<C>(k)], zc = pen[sm_idx<C>((N - k) & (N - 1))];
     C *dst = out + ((size_t)f * NN + row0 + 2 * p) * NX;
-    dst[k] = c_store(c_scale(C{z.re + zc.re, z.im - zc.im}, (typename scale_of<C>::type)0.5));
-    dst[NX + k] = c_store(c_scale(C{z.im + zc.im, zc.re - z.re}, (typename scale_of<C>::type)0.5));
+    dst[k] = c_store(half(C{z.re + zc.re, z.im - zc.im}));
+    dst[NX + k] = c_store(half(C{z.im + zc.im, zc.re - z.re}));
   }
 }
 
@@ -591,13 +599,13 @@ __global__ void __launch_bounds__(kMaxThreads) get_x_kernel(const C *__restrict_
       pen[sm_idx<C>(N - k)] = C{x0.re + x1.im, x1.re - x0.im};
     }
   }
-  for (int q = threadIdx.x; q < nf * PAIRS * (N - 2 * KT - 1); q += nthr) {
-    const int z = q % (N - 2 * KT - 1);
-    const int r = q / (N - 2 * KT - 1);
-    sm[r * P + sm_idx<C>(KT + 1 + z)] = C{0, 0};
+  constexpr int NZ = pencil_zero_count<N>();
+  for (unsigned q = threadIdx.x; q < (unsigned)(nf * PAIRS * NZ); q += nthr) {
+    const unsigned z = q % NZ, r = q / NZ;
+    sm[r * P + sm_at<C>(pencil_zero<N>(z))] = C{0, 0};
   }
   __syncthreads();
-  fft_pencils<N, +1, 8>(nf * PAIRS, [&](int id) { return sm + id * P; }, tw);
+  fft_pencils<N, +1, 8, std::is_same<C, cplx64>::value>(nf * PAIRS, [&](int id) { return sm + id * P; }, tw);
   for (int q = threadIdx.x; q < nf * PAIRS * N; q += nthr) {
     const int j = q % N;
     const int r = q / N;
@@ -640,10 +648,10 @@ __global__ void __launch_bounds__(kMaxThreads) diag_x_kernel(const cplx64 *__res
       pen[sm_idx<cplx64>(N - k)] = cplx64{x0.re + x1.im, x1.re - x0.im};
     }
   }
-  for (int q = threadIdx.x; q < 7 * PAIRS * (N - 2 * KT - 1); q += nthr) {
-    const int z = q % (N - 2 * KT - 1);
-    const int r = q / (N - 2 * KT - 1);
-    sm[r * P + sm_idx<cplx64>(KT + 1 + z)] = cplx64{0.0, 0.0};
+  constexpr int NZ = pencil_zero_count<N>();
+  for (unsigned q = threadIdx.x; q < (unsigned)(7 * PAIRS * NZ); q += nthr) {
+    const unsigned z = q % NZ, r = q / NZ;
+    sm[r * P + sm_at<cplx64>(pencil_zero<N>(z))] = cplx64{0.0, 0.0};
   }
   __syncthreads();
   fft_pencils<N, +1, 8>(7 * PAIRS, [&](int id) { return sm + id * P; }, tw);
