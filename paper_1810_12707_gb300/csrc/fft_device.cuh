@@ -257,6 +257,24 @@ __device__ __forceinline__ const W *tw_at(const W *table, unsigned kt, int r) {
   }
 }
 
+__device__ __forceinline__ cplx64 tw_load(const cplx64 *p) {
+  cplx64 v;
+  asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.re), "=d"(v.im) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ TwFx tw_load(const TwFx *p) {
+  TwFx v;
+  asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.ch), "=r"(v.cl), "=r"(v.sh), "=r"(v.sl)
+               : "l"(p));
+  return v;
+}
+__device__ __forceinline__ cplx32 tw_load(const cplx32 *p) {
+  cplx32 v;
+  asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.re), "=f"(v.im) : "l"(p));
+  return v;
+}
+
 // The value of x, opaque to the optimiser: index arithmetic derived from it cannot be hoisted out
 // of a persistent loop and kept live (in registers or spilled) across iterations.
 __device__ __forceinline__ int launder(int x) {
