@@ -513,8 +513,10 @@ __host__ __device__ constexpr int fft_tpp() { return tpp_for<N, fft_vpt<C>()>();
 // `active == false` only take part in the barriers.  The caller separates the transform from the
 // preceding writes and the following reads of the pencil with a block barrier.
 // TWG: `tw` points to shared memory (double-float only).
-template <int N, int DIR, int NS, typename C, int VPT, bool ZP, bool TWG = false>
-__device__ __forceinline__ void stockham_stages(C *buf, int t, bool active, const C *__restrict__ tw) {
+// REG: the last stage leaves its results in `out` instead of the pencil: out[q] = X[t + q N/VPT].
+template <int N, int DIR, int NS, typename C, int VPT, bool ZP, bool TWG = false, bool REG = false>
+__device__ __forceinline__ void stockham_stages(C *buf, int t, bool active, const C *__restrict__ tw,
+                                                C *out = nullptr) {
   if constexpr (NS < N) {
     static_assert(VPT == 8 || (VPT == 16 && sizeof(C) == 8), "radix 16 is an FP32 option");
     constexpr int R = (N / NS >= VPT) ? VPT : N / NS;
@@ -574,13 +576,18 @@ __device__ __forceinline__ void stockham_stages(C *buf, int t, bool active, cons
         } else {
           dft_small<R, DIR, C>(v + b * R);
         }
-        C *wp = buf + sm_at<C>((j - k) * R + k);
+        if constexpr (REG && NS * R == N) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) wp[sm_idx<C>(r * NS)] = v[b * R + r];
+          for (int r = 0; r < R; ++r) out[b + NB * r] = v[b * R + r];
+        } else {
+          C *wp = buf + sm_at<C>((j - k) * R + k);
+#pragma unroll
+          for (int r = 0; r < R; ++r) wp[sm_idx<C>(r * NS)] = v[b * R + r];
+        }
       }
     }
-    group_sync<TPP>();
-    stockham_stages<N, DIR, NS * R, C, VPT, false, TWG>(buf, t, active, tw);
+    if constexpr (!(REG && NS * R == N)) group_sync<TPP>();
+    stockham_stages<N, DIR, NS * R, C, VPT, false, TWG, REG>(buf, t, active, tw, out);
   }
 }
 
@@ -592,11 +599,12 @@ __device__ __forceinline__ void stockham_stages(C *buf, int t, bool active, cons
 // 256^3 step 14.75 -> 4.97.  The exponent's reduction adds no barrier: a group of
 // more than a warp leaves its warps' parts in shared memory before the barrier that the first
 // stage has between its reads and its writes anyway.  It depends on the group's threads only, so
-// a pencil's results are the same bits in every kernel and at every tile width.
+// a pencil's results are the same bits in every kernel with the same DP and at every tile width.
 // DP: the results' conversion runs on the FP64 pipe; `scale2`: they are scaled by 2^scale2.
-template <int N, int DIR, int NS, bool DP>
+// REG: the last stage leaves its fixed-point results in `out`, as in stockham_stages.
+template <int N, int DIR, int NS, bool DP, bool REG = false>
 __device__ __forceinline__ void fx_stages(cfx *buf, int t, bool active, const TwFx *__restrict__ tw, const FxScale &sc,
-                                          int left, int scale2) {
+                                          int left, int scale2, cfx *out = nullptr) {
   constexpr int R = N / NS >= 8 ? 8 : N / NS;
   constexpr int NB = 8 / R;
   constexpr int TPP = tpp_for<N, 8>();
@@ -620,6 +628,13 @@ __device__ __forceinline__ void fx_stages(cfx *buf, int t, bool active, const Tw
     }
   }
   group_sync<TPP>();
+  if constexpr (REG && NS * R == N) {
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int r = 0; r < R; ++r) out[b + NB * r] = v[b * R + r];
+    return;
+  }
   if (active) {
     const uint32_t be = sc.ek + (uint32_t)(sc.shift + scale2) + 1u;
 #pragma unroll
@@ -644,45 +659,24 @@ __device__ __forceinline__ void fx_stages(cfx *buf, int t, bool active, const Tw
     }
   }
   group_sync<TPP>();
-  if constexpr (NS * R < N) fx_stages<N, DIR, NS * R, DP>(buf, t, active, tw, sc, left - s, scale2);
+  if constexpr (NS * R < N) fx_stages<N, DIR, NS * R, DP, REG>(buf, t, active, tw, sc, left - s, scale2, out);
 }
 
-template <int N, int DIR, bool ZP, bool DP = false>
-__device__ __forceinline__ void fx_pencil_fft(cplx64 *buf, int t, bool active, const TwFx *__restrict__ tw,
-                                              int scale2 = 0) {
+// The pencil's scale from every thread's share of its values: `size(m)` is the thread's sum of their
+// sizes in units of 2^(m - 1043) (fx_size), `m` its largest biased exponent.  Holds one group barrier
+// if SYNC or if the group is more than a warp.
+template <int N, bool SYNC, typename Size>
+__device__ __forceinline__ FxScale fx_group_scale(uint32_t m, Size size) {
   constexpr int TPP = tpp_for<N, 8>();
   constexpr int LOG2G = TPP == 128 ? 7 : TPP == 64 ? 6 : TPP == 32 ? 5 : TPP == 16 ? 4 : TPP == 8 ? 3 : TPP == 4 ? 2 : 1;
-  constexpr int K = (N - 1) / 3;
-  static_assert(!ZP || (3 * (N / 8) > K && 5 * (N / 8) - 1 < N - K),
-                "inputs 3 and 4 of the first stage must lie in the 2/3-rule gap");
   __shared__ FxPart part[32];  // one entry per warp, for groups of more than one
-  cplx64 x[8];
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    x[r] = cplx64{0.0, 0.0};
-    if (!(ZP && (r == 3 || r == 4)) && active)
-      x[r] = TPP % sm_pad<cplx64>() == 0 ? buf[sm_at<cplx64>((unsigned)t) + sm_idx<cplx64>(r * TPP)]
-                                         : buf[sm_at<cplx64>((unsigned)(t + r * TPP))];
-  }
-  uint32_t m = 0u;
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    if (ZP && (r == 3 || r == 4)) continue;
-    m = max(m, max(fx_hi(x[r].re) & 0x7fffffffu, fx_hi(x[r].im) & 0x7fffffffu));
-  }
-  m >>= 20;
   if constexpr (TPP >= 32) {
     m = __reduce_max_sync(0xffffffffu, m);
   } else {
 #pragma unroll
     for (int o = TPP / 2; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(existing_lanes(), m, o));
   }
-  FxPart p = {m, 0u, 0u};
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    if (ZP && (r == 3 || r == 4)) continue;
-    p.a += fx_size(fx_hi(x[r].re), m) + fx_size(fx_hi(x[r].im), m);
-  }
+  FxPart p = {m, size(m), 0u};
   p.t = (p.a >> 3) + 1u;
   if constexpr (TPP >= 32) {
     p.a = __reduce_max_sync(0xffffffffu, p.a);
@@ -697,14 +691,45 @@ __device__ __forceinline__ void fx_pencil_fft(cplx64 *buf, int t, bool active, c
   if constexpr (TPP > 32) {
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = p;
   }
-  group_sync<TPP>();
+  if constexpr (SYNC || TPP > 32) group_sync<TPP>();
   if constexpr (TPP > 32) {
     const int w0 = (threadIdx.x / TPP) * (TPP / 32);
     p = part[w0];
 #pragma unroll
     for (int i = 1; i < TPP / 32; ++i) p = fx_merge(p, part[w0 + i]);
   }
-  const FxScale sc = fx_scale(p, LOG2G);
+  return fx_scale(p, LOG2G);
+}
+
+// The transform of the doubles in `buf`: results in the pencil as doubles, or (REG) in `out` as
+// fixed-point values of scale `sc`.
+template <int N, int DIR, bool ZP, bool DP = false, bool REG = false>
+__device__ __forceinline__ void fx_pencil_fft(cplx64 *buf, int t, bool active, const TwFx *__restrict__ tw,
+                                              int scale2 = 0, cfx *out = nullptr, FxScale *out_scale = nullptr) {
+  constexpr int TPP = tpp_for<N, 8>();
+  constexpr int K = (N - 1) / 3;
+  static_assert(!ZP || (3 * (N / 8) > K && 5 * (N / 8) - 1 < N - K),
+                "inputs 3 and 4 of the first stage must lie in the 2/3-rule gap");
+  cplx64 x[8];
+  uint32_t m = 0u;
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    x[r] = cplx64{0.0, 0.0};
+    if (ZP && (r == 3 || r == 4)) continue;
+    if (active)
+      x[r] = TPP % sm_pad<cplx64>() == 0 ? buf[sm_at<cplx64>((unsigned)t) + sm_idx<cplx64>(r * TPP)]
+                                         : buf[sm_at<cplx64>((unsigned)(t + r * TPP))];
+    m = max(m, max(fx_hi(x[r].re) & 0x7fffffffu, fx_hi(x[r].im) & 0x7fffffffu));
+  }
+  const FxScale sc = fx_group_scale<N, true>(m >> 20, [&](uint32_t mm) {
+    uint32_t a = 0u;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      if (ZP && (r == 3 || r == 4)) continue;
+      a += fx_size(fx_hi(x[r].re), mm) + fx_size(fx_hi(x[r].im), mm);
+    }
+    return a;
+  });
   cfx *fb = reinterpret_cast<cfx *>(buf);
   if (active) {
     cfx v[8];
@@ -719,7 +744,8 @@ __device__ __forceinline__ void fx_pencil_fft(cplx64 *buf, int t, bool active, c
     for (int r = 0; r < 8; ++r) fb[9u * (unsigned)t + r] = v[r];
   }
   group_sync<TPP>();
-  fx_stages<N, DIR, 8, DP>(fb, t, active, tw, sc, sc.shift, scale2);
+  fx_stages<N, DIR, 8, DP, REG>(fb, t, active, tw, sc, sc.shift, scale2, out);
+  if constexpr (REG) *out_scale = sc;
 }
 
 // `t` in [0, N / VPT): the thread's index within its pencil's group.  ZP: the pencil is
@@ -745,6 +771,180 @@ __device__ __forceinline__ void pencil_fft(C *buf, int t, bool active, const TW 
     fx_pencil_fft<N, DIR, ZP, DP>(buf, t, active, tw, scale2);
   } else {
     stockham_stages<N, DIR, 1, C, VPT, ZP, TWG>(buf, t, active, tw);
+  }
+}
+
+// ---- x passes: two real rows as one pencil, straight from and to their half spectra ----
+// Thread t of a group owns the half-spectrum values k = t + i TPP, i < row_vals: in the pencil
+// Z[k] = X0[k] + i X1[k] they are inputs i of its first-stage butterfly, and after a forward
+// transform the last stage leaves Z[k] in its registers.  Only the mirrored values Z[N-k], which
+// belong to thread TPP - t, cross through shared memory: 3 of a butterfly's 8 values (6 of 16)
+// instead of all of them twice, with no zeros to write and no index arithmetic per value.
+template <int N, int VPT>
+__host__ __device__ constexpr int row_vals() {
+  return ((N - 1) / 3 + tpp_for<N, VPT>()) / tpp_for<N, VPT>();  // ceil(NX / TPP)
+}
+template <int N, typename C, int VPT>
+struct RowPair {
+  static constexpr int NI = row_vals<N, VPT>(), TPP = tpp_for<N, VPT>(), NX = (N - 1) / 3 + 1;
+  static_assert((VPT == 8 && NI == 3) || (VPT == 16 && NI == 6), "the kept values are a butterfly's outer inputs");
+  static constexpr bool kConst = TPP % sm_pad<C>() == 0;
+  C x0[NI], x1[NI];
+
+  __device__ __forceinline__ static bool kept(int t, int i) { return (i + 1) * TPP <= NX || t + i * TPP < NX; }
+  // rows at src and src + NX (zeros beyond K and for an inactive group)
+  __device__ __forceinline__ void load(const C *__restrict__ src, int t, bool active) {
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      x0[i] = x1[i] = C{0, 0};
+      if (active && kept(t, i)) {
+        x0[i] = src[t + i * TPP];
+        x1[i] = src[NX + t + i * TPP];
+      }
+    }
+  }
+  // pencil element N - (t + i TPP)
+  template <typename E>
+  __device__ __forceinline__ static E *mirror(E *buf, int t, int i) {
+    if constexpr (kConst) return buf + sm_at<C>((unsigned)(N - t)) - sm_idx<C>(i * TPP);
+    else return buf + sm_at<C>((unsigned)(N - t - i * TPP));
+  }
+  // pencil element t + r TPP
+  template <typename E>
+  __device__ __forceinline__ static E *own(E *buf, int t, int r) {
+    if constexpr (kConst) return buf + sm_at<C>((unsigned)t) + sm_idx<C>(r * TPP);
+    else return buf + sm_at<C>((unsigned)(t + r * TPP));
+  }
+  // whether element t + r TPP, r >= VPT - NI, is a mirrored kept value
+  __device__ __forceinline__ static bool mirrored(int t, int r) { return N - t - r * TPP < NX; }
+};
+
+// Inverse transform of a row pair into the pencil `buf` (real part: row 0, imaginary part: row 1).
+// DP as in pencil_fft.
+template <int N, typename C, int VPT, bool DP, typename TW>
+__device__ __forceinline__ void rows_inverse(C *buf, int t, bool active, RowPair<N, C, VPT> &x,
+                                             const TW *__restrict__ tw) {
+  using RP = RowPair<N, C, VPT>;
+  constexpr int NI = RP::NI, TPP = RP::TPP;
+  if constexpr (std::is_same<TW, TwFx>::value) {
+    if (t == 0) x.x0[0].im = x.x1[0].im = 0.0;  // k = 0: the Hermitian part
+    uint32_t m = 0u;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      m = max(m, max(fx_hi(x.x0[i].re) & 0x7fffffffu, fx_hi(x.x0[i].im) & 0x7fffffffu));
+      m = max(m, max(fx_hi(x.x1[i].re) & 0x7fffffffu, fx_hi(x.x1[i].im) & 0x7fffffffu));
+    }
+    // a thread's values bound its own inputs of the first stage and their mirror images alike
+    const FxScale sc = fx_group_scale<N, false>(m >> 20, [&](uint32_t mm) {
+      uint32_t a = 0u;
+#pragma unroll
+      for (int i = 0; i < NI; ++i)
+        a += fx_size(fx_hi(x.x0[i].re), mm) + fx_size(fx_hi(x.x0[i].im), mm) + fx_size(fx_hi(x.x1[i].re), mm) +
+             fx_size(fx_hi(x.x1[i].im), mm);
+      return 2u * a;
+    });
+    cfx *fb = reinterpret_cast<cfx *>(buf);
+    cfx v[8];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const int64_t a = fx_from_double(fx_hi(x.x0[i].re), fx_lo(x.x0[i].re), sc.ek);
+      const int64_t b = fx_from_double(fx_hi(x.x0[i].im), fx_lo(x.x0[i].im), sc.ek);
+      const int64_t c = fx_from_double(fx_hi(x.x1[i].re), fx_lo(x.x1[i].re), sc.ek);
+      const int64_t d = fx_from_double(fx_hi(x.x1[i].im), fx_lo(x.x1[i].im), sc.ek);
+      v[i] = cfx{a - d, b + c};
+      if (active && RP::kept(t, i) && (i > 0 || t > 0)) *RP::mirror(fb, t, i) = cfx{a + d, c - b};
+    }
+    group_sync<TPP>();
+    if (active) {
+#pragma unroll
+      for (int r = 8 - NI; r < 8; ++r) {
+        v[r] = cfx{0, 0};
+        if (RP::mirrored(t, r)) v[r] = *RP::own(fb, t, r);
+      }
+      fx_dft8<+1, true>(v);
+    }
+    group_sync<TPP>();
+    if (active) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) fb[9u * (unsigned)t + r] = v[r];
+    }
+    group_sync<TPP>();
+    fx_stages<N, +1, 8, DP>(fb, t, active, tw, sc, sc.shift, 0);
+  } else {
+    C v[VPT];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const C x0 = x.x0[i], x1 = x.x1[i];
+      v[i] = C{x0.re - x1.im, x0.im + x1.re};
+      if (i == 0 && t == 0) v[0] = C{x0.re, x1.re};  // k = 0: the Hermitian part
+      if (active && RP::kept(t, i) && (i > 0 || t > 0)) *RP::mirror(buf, t, i) = C{x0.re + x1.im, x1.re - x0.im};
+    }
+    group_sync<TPP>();
+    if (active) {
+#pragma unroll
+      for (int r = NI; r < VPT; ++r) {
+        v[r] = C{0, 0};
+        if (r >= VPT - NI && RP::mirrored(t, r)) v[r] = *RP::own(buf, t, r);
+      }
+      if constexpr (VPT == 16) dft16<+1, C, true>(v);
+      else dft8_first_fma<+1, true>(v);
+    }
+    group_sync<TPP>();
+    if (active) {
+      C *wp = buf + sm_at<C>((unsigned)(t * VPT));
+#pragma unroll
+      for (int r = 0; r < VPT; ++r) wp[sm_idx<C>(r)] = v[r];
+    }
+    group_sync<TPP>();
+    stockham_stages<N, +1, VPT, C, VPT, false>(buf, t, active, tw);
+  }
+}
+
+// Forward transform of the pencil `buf` and the half spectra of its two rows, doubled (the split's
+// factor 1/2 is left out; fixed point: scaled by 2^scale2), to dst and dst + NX.
+template <int N, typename C, int VPT, bool DP, typename TW, typename Post>
+__device__ __forceinline__ void rows_forward(C *buf, int t, bool active, C *__restrict__ dst,
+                                             const TW *__restrict__ tw, int scale2, Post post) {
+  using RP = RowPair<N, C, VPT>;
+  constexpr int NI = RP::NI, TPP = RP::TPP, NX = RP::NX;
+  constexpr bool kFx = std::is_same<TW, TwFx>::value;
+  using E = typename std::conditional<kFx, cfx, C>::type;
+  E *eb = reinterpret_cast<E *>(buf);
+  E z[VPT];
+  FxScale sc{};
+  if constexpr (kFx) {
+    fx_pencil_fft<N, -1, false, DP, true>(buf, t, active, tw, 0, z, &sc);
+  } else {
+    stockham_stages<N, -1, 1, C, VPT, false, false, true>(buf, t, active, tw, z);
+  }
+  // (the last stage has a barrier after its reads)
+  if (active) {
+#pragma unroll
+    for (int r = VPT - NI; r < VPT; ++r)
+      if (RP::mirrored(t, r)) *RP::own(eb, t, r) = z[r];
+  }
+  group_sync<TPP>();
+  if (active) {
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      if (!RP::kept(t, i)) continue;
+      E zc = z[0];
+      if (i > 0 || t > 0) zc = *RP::mirror(eb, t, i);
+      const E r0 = {z[i].re + zc.re, z[i].im - zc.im}, r1 = {z[i].im + zc.im, zc.re - z[i].re};
+      C y0, y1;
+      if constexpr (kFx) {
+        const uint32_t be = sc.ek + (uint32_t)(sc.shift + scale2) + 1u;
+        auto out = [&](int64_t v) { return DP ? fx_to_double_dp(v, be) : fx_to_double(v, be); };
+        y0 = C{out(r0.re), out(r0.im)};
+        y1 = C{out(r1.re), out(r1.im)};
+        if (sc.bad) y0.re = y0.im = y1.re = y1.im = fx_double(0x7ff80000u, 0u);
+      } else {
+        y0 = post(r0);
+        y1 = post(r1);
+      }
+      dst[t + i * TPP] = y0;
+      dst[NX + t + i * TPP] = y1;
+    }
   }
 }
 

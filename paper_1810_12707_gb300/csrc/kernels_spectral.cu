@@ -851,7 +851,8 @@ __global__ void __launch_bounds__(fused_max_threads<N, VPT>(), (fused_max_thread
   const int pencil = threadIdx.x / TPP;
   const int t = threadIdx.x - pencil * TPP;
   const bool active = q0 + (pencil & (tc - 1)) < COLS;
-  pencil_fft<N, +1, C, VPT, true>(sm + (active ? pencil : 0) * P, t, active, tw);
+  // DP as in the inverse z pass, whose bits these are
+  pencil_fft<N, +1, C, VPT, true, false, std::is_same<C, cplx64>::value>(sm + (active ? pencil : 0) * P, t, active, tw);
   __syncthreads();
 
   // 3. rows z of the next inverse y pass's input, TC consecutive columns per row

@@ -64,6 +64,31 @@ constexpr int flux_min_blocks() {
   return b < 1 ? 1 : b;
 }
 
+// Whether a group loads its next row pair before it transforms one: not where the registers that
+// holds cost more than the loads' latency (double-float 256^3 1.85 -> 1.81 ms, 512^3 17.6 -> 16.4; FP64
+// 512^3 20.5 -> 19.8, but 256^3 2.31 -> 2.33).
+template <int N, typename C>
+constexpr bool flux_ahead() { return std::is_same<C, cplx64>::value ? N != 512 : !std::is_same<C, cdf>::value; }
+
+// 1 / x from the hardware's approximation r0 (relative error e, about 2^-20) by Householder's
+// iteration of third order, r0 (1 + e + e^2) with e = 1 - x r0: the neglected e^3 is below 2^-57, so
+// only the last fused multiply-add rounds.  Four FP64 instructions where the division takes about
+// twice as many.  Not finite for x = 0, infinite or NaN (a NaN).
+__device__ __forceinline__ double rcp3(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// |x| as an FP32 number from the high word alone, truncated (at most 2^-20 relative below |x|);
+// infinite from 2^128 on and for a NaN, 0 below 2^-126.  Integer instructions: a conversion costs
+// as much as an FP64 multiplication.
+__device__ __forceinline__ float float_below(double x) {
+  const int h = (__double2hiint(x) & 0x7fffffff) - 0x38000000;
+  return __int_as_float(min(max(h, 0), 0x0ff00000) << 3);
+}
+
 // Run the FFT of `np` pencils (pencil id -> shared-memory pointer `ptr(id)`) with every group of
 // N/VPT threads of the block taking one pencil at a time.  Each pencil is touched by its group only,
 // so the stages synchronise per group; one block barrier closes the whole transform.
@@ -113,37 +138,33 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
   // the launch uses exactly this many threads, so every loop below has a constant trip count
   constexpr int nthr = flux_threads<N, C>();
 
-  // 1. load and pack the 7 state fields: pencil (p, f) at sm + (p * 12 + f) * P.  Unrolled: all
-  // of a thread's loads are issued before the first shared-memory store.
-  constexpr int NLD = 7 * PAIRS * NX;
-#pragma unroll
-  for (int q0 = 0; q0 < NLD; q0 += nthr) {
-    const int q = q0 + (int)threadIdx.x;
-    if (q < NLD) {
-      const int k = q % NX;
-      const int r = q / NX;
-      const int f = r % 7, p = r / 7;
-      const C *src = in + ((size_t)(inst * 7 + f) * NN + row0 + 2 * p) * NX;
-      C *pen = sm + (p * 12 + f) * P;
-      const C x0 = src[k], x1 = src[NX + k];
-      if (k == 0) {
-        pen[0] = C{x0.re, x1.re};
+  // 1. inverse transforms of the 7 state fields: pencil (p, f) at sm + (p * 12 + f) * P, each by one
+  // group, which loads its next row pair while it transforms one
+  constexpr int VPT = flux_vpt<N, C>(), TPP = tpp_for<N, VPT>(), G = nthr / TPP;
+  const int g = threadIdx.x / TPP, t = threadIdx.x - g * TPP;
+  {
+    auto src = [&](int id) {
+      return in + ((size_t)(inst * 7 + id % 7) * NN + row0 + 2 * (id / 7)) * NX;
+    };
+    RowPair<N, C, VPT> x;
+    if constexpr (flux_ahead<N, C>()) x.load(src(g < 7 * PAIRS ? g : 0), t, g < 7 * PAIRS);
+#pragma unroll 1
+    for (int base = 0; base < 7 * PAIRS; base += G) {
+      const int id = base + g;
+      const bool active = id < 7 * PAIRS, more = id + G < 7 * PAIRS;
+      C *pen = sm + (active ? (id / 7) * 12 + id % 7 : 0) * P;
+      if constexpr (flux_ahead<N, C>()) {
+        RowPair<N, C, VPT> next;
+        if (base + G < 7 * PAIRS) next.load(src(more ? id + G : 0), t, more);
+        rows_inverse<N, C, VPT, false>(pen, t, active, x, tw);
+        x = next;
       } else {
-        pen[sm_idx<C>(k)] = C{x0.re - x1.im, x0.im + x1.re};
-        pen[sm_idx<C>(N - k)] = C{x0.re + x1.im, x1.re - x0.im};
+        x.load(src(active ? id : 0), t, active);
+        rows_inverse<N, C, VPT, false>(pen, t, active, x, tw);
       }
     }
   }
-  constexpr int NZ = pencil_zero_count<N>();
-  for (unsigned q = threadIdx.x; q < (unsigned)(7 * PAIRS * NZ); q += nthr) {
-    const unsigned z = q % NZ, r = q / NZ;
-    const unsigned f = r % 7, p = r / 7;
-    sm[(p * 12 + f) * P + sm_at<C>(pencil_zero<N>(z))] = C{0, 0};
-  }
   __syncthreads();
-
-  // 2. inverse transforms of the 7 fields
-  fft_pencils<N, +1, (flux_vpt<N, C>())>(7 * PAIRS, [&](int id) { return sm + ((id / 7) * 12 + id % 7) * P; }, tw);
 
   // 3. products on the grid (real part: row 0, imaginary part: row 1)
   constexpr bool kDF = std::is_same<C, cdf>::value;
@@ -151,23 +172,24 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
   SM smax = 0;
   // FP64 and double-float: the maximum that blocks of this pass have already published is a
   // lower bound of the pass's maximum.  A point whose FP32 estimate of |u| + c_f lies below
-  // `screen` (that bound less 1e-6 relative and 1e-18 absolute, above the estimate's worst error
-  // of about 3e-7 relative) cannot raise it, so its exact speed (two FP64 square roots) is not
-  // formed.  The pass still yields the exact maximum, whichever blocks ran first; a NaN or an
-  // infinite estimate always takes the exact path.
+  // `screen` (that bound less 3e-6 relative and 1e-18 absolute, above the estimate's worst error:
+  // 3e-7 relative from FP32 sums and roots, and in FP64 1e-6 from the truncated operands) cannot
+  // raise it, so its exact speed (two FP64 square roots) is not formed.  The pass still yields the
+  // exact maximum, whichever blocks ran first; a NaN, an infinite estimate or a negative density
+  // always takes the exact path.
   float screen = 0.f;
   if constexpr (sizeof(SM) == 8) {
     const double lb = __longlong_as_double((long long)*reinterpret_cast<volatile unsigned long long *>(smax_bits + inst));
-    screen = (float)(lb * (1.0 - 1e-6) - 1e-18);
+    screen = (float)(lb * (1.0 - 3e-6) - 1e-18);
   }
   if constexpr (kDF) {
     // double-float products.  The grid values leave the inverse transforms unnormalised; near a
     // zero of a field (a stagnation point) their low part can exceed the high part, and the
     // square of such a pair, which drops lo^2, can come out negative.  So they are renormalised
     // first (then |lo| <= ulp(hi) / 2 and every square is >= 0), as are the velocity components
-    // before the speed is formed; the speed's squares are renormalised too, so their high parts
-    // are the FP32 roundings the screening estimate assumes, and the exact speed is taken in FP64
-    // from the double-float squares.
+    // before the exact speed is formed.  The screening estimate takes the high parts alone (FP32
+    // products of normalised values, within an ulp); the exact speed is taken in FP64 from the
+    // double-float squares, at the points that pass.
     const double csd = phys[inst].cs;
     const dfr cs2 = dfr_from_double(csd * csd);
     for (int q = threadIdx.x; q < PAIRS * N; q += nthr) {
@@ -212,9 +234,10 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
         bd[2 * 9 * P + h] = ux;
         bd[2 * 10 * P + h] = uy;
         bd[2 * 11 * P + h] = uz;
-        const dfr nx = dfr_norm(ux), ny = dfr_norm(uy), nz = dfr_norm(uz);
-        const dfr u2 = dfr_norm(nx * nx + ny * ny + nz * nz), c2 = dfr_norm(cs2 + b2 * ir);
-        if (!(sqrtf(u2.hi) + sqrtf(c2.hi) < screen)) {
+        const float u2f = ux.hi * ux.hi + uy.hi * uy.hi + uz.hi * uz.hi, c2f = cs2.hi + b2.hi * ir.hi;
+        if (!(sqrtf(u2f) + sqrtf(c2f) < screen)) {
+          const dfr nx = dfr_norm(ux), ny = dfr_norm(uy), nz = dfr_norm(uz);
+          const dfr u2 = dfr_norm(nx * nx + ny * ny + nz * nz), c2 = dfr_norm(cs2 + b2 * ir);
           const double s = sqrt(dfr_to_double(u2)) + sqrt(dfr_to_double(c2));
           smax = (s != s || s > smax) ? s : smax;  // keeps a NaN once seen
         }
@@ -222,6 +245,7 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
     }
   } else {
   const R cs2 = (R)(phys[inst].cs * phys[inst].cs);
+  const float cs2f = (float)cs2;
   for (int q = threadIdx.x; q < PAIRS * N; q += nthr) {
     const int p = q / N, j = q - p * N;
     C *b = sm + p * 12 * P + sm_idx<C>(j);
@@ -247,7 +271,9 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
       const R rho = v[h][0];
       const R mx = v[h][1], my = v[h][2], mz = v[h][3];
       const R bx = v[h][4], by = v[h][5], bz = v[h][6];
-      const R ir = (R)1 / rho;
+      R ir;
+      if constexpr (sizeof(R) == 8) ir = rcp3(rho);
+      else ir = (R)1 / rho;
       const R ux = mx * ir, uy = my * ir, uz = mz * ir;
       const R b2 = bx * bx + by * by + bz * bz;
       const R hb = (R)0.5 * b2;
@@ -264,14 +290,15 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
       bd[2 * 9 * P + h] = ux;
       bd[2 * 10 * P + h] = uy;
       bd[2 * 11 * P + h] = uz;
-      const R u2 = ux * ux + uy * uy + uz * uz, c2 = cs2 + b2 * ir;
       if constexpr (sizeof(R) == 8) {
-        if (!(sqrtf((float)u2) + sqrtf((float)c2) < screen)) {
-          const R s = sqrt(u2) + sqrt(c2);
+        const float fx = float_below(ux), fy = float_below(uy), fz = float_below(uz);
+        const float u2f = fx * fx + fy * fy + fz * fz, c2f = cs2f + float_below(b2) * float_below(ir);
+        if (!(sqrtf(u2f) + sqrtf(c2f) < screen) || __double2hiint(ir) < 0) {
+          const R s = sqrt(ux * ux + uy * uy + uz * uz) + sqrt(cs2 + b2 * ir);
           smax = (s != s || s > smax) ? s : smax;  // keeps a NaN once seen
         }
       } else {
-        const R s = sqrt(u2) + sqrt(c2);
+        const R s = sqrt(ux * ux + uy * uy + uz * uz) + sqrt(cs2 + b2 * ir);
         smax = (s != s || s > smax) ? s : smax;
       }
     }
@@ -279,19 +306,15 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
   }
   __syncthreads();
 
-  // 4. forward transforms of the 12 products
-  fft_pencils<N, -1, (flux_vpt<N, C>())>(12 * PAIRS, [&](int id) { return sm + id * P; }, tw);
-
-  // 5. unpack and store the kept half spectra
-  for (int q = threadIdx.x; q < 12 * PAIRS * NX; q += nthr) {
-    const int k = q % NX;
-    const int r = q / NX;
-    const int f = r % 12, p = r / 12;
-    const C *pen = sm + (p * 12 + f) * P;
-    const C z = pen[sm_idx<C>(k)], zc = pen[sm_idx<C>((N - k) & (N - 1))];
-    C *dst = out + ((size_t)(inst * 12 + f) * NN + row0 + 2 * p) * NX;
-    dst[k] = c_store(C{z.re + zc.re, z.im - zc.im});
-    dst[NX + k] = c_store(C{z.im + zc.im, zc.re - z.re});
+  // 4. forward transforms of the 12 products, their kept half spectra to memory
+#pragma unroll 1
+  for (int base = 0; base < 12 * PAIRS; base += G) {
+    const int id = base + g;
+    const bool active = id < 12 * PAIRS;
+    const int f = id % 12, p = id / 12;
+    rows_forward<N, C, VPT, false>(sm + (active ? id : 0) * P, t, active,
+                                   out + ((size_t)(inst * 12 + f) * NN + row0 + 2 * p) * NX, tw, 0,
+                                   [](C v) { return c_store(v); });
   }
 
   const SM m = block_nan_max(smax, reinterpret_cast<SM *>(red));
