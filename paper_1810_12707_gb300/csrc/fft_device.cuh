@@ -701,24 +701,21 @@ __device__ __forceinline__ FxScale fx_group_scale(uint32_t m, Size size) {
   return fx_scale(p, LOG2G);
 }
 
-// The transform of the doubles in `buf`: results in the pencil as doubles, or (REG) in `out` as
-// fixed-point values of scale `sc`.
+// The transform of the doubles x[r] = element t + r N/8 of each thread of the group: results in the
+// pencil `buf` as doubles, or (REG) in `out` as fixed-point values of scale `sc`.  Nothing is read
+// from `buf` before the group's first barrier.
 template <int N, int DIR, bool ZP, bool DP = false, bool REG = false>
-__device__ __forceinline__ void fx_pencil_fft(cplx64 *buf, int t, bool active, const TwFx *__restrict__ tw,
-                                              int scale2 = 0, cfx *out = nullptr, FxScale *out_scale = nullptr) {
+__device__ __forceinline__ void fx_fft_from(const cplx64 *x, cplx64 *buf, int t, bool active,
+                                            const TwFx *__restrict__ tw, int scale2 = 0, cfx *out = nullptr,
+                                            FxScale *out_scale = nullptr) {
   constexpr int TPP = tpp_for<N, 8>();
   constexpr int K = (N - 1) / 3;
   static_assert(!ZP || (3 * (N / 8) > K && 5 * (N / 8) - 1 < N - K),
                 "inputs 3 and 4 of the first stage must lie in the 2/3-rule gap");
-  cplx64 x[8];
   uint32_t m = 0u;
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
-    x[r] = cplx64{0.0, 0.0};
     if (ZP && (r == 3 || r == 4)) continue;
-    if (active)
-      x[r] = TPP % sm_pad<cplx64>() == 0 ? buf[sm_at<cplx64>((unsigned)t) + sm_idx<cplx64>(r * TPP)]
-                                         : buf[sm_at<cplx64>((unsigned)(t + r * TPP))];
     m = max(m, max(fx_hi(x[r].re) & 0x7fffffffu, fx_hi(x[r].im) & 0x7fffffffu));
   }
   const FxScale sc = fx_group_scale<N, true>(m >> 20, [&](uint32_t mm) {
@@ -746,6 +743,22 @@ __device__ __forceinline__ void fx_pencil_fft(cplx64 *buf, int t, bool active, c
   group_sync<TPP>();
   fx_stages<N, DIR, 8, DP, REG>(fb, t, active, tw, sc, sc.shift, scale2, out);
   if constexpr (REG) *out_scale = sc;
+}
+
+// The same of the doubles in the pencil `buf`.
+template <int N, int DIR, bool ZP, bool DP = false, bool REG = false>
+__device__ __forceinline__ void fx_pencil_fft(cplx64 *buf, int t, bool active, const TwFx *__restrict__ tw,
+                                              int scale2 = 0, cfx *out = nullptr, FxScale *out_scale = nullptr) {
+  constexpr int TPP = tpp_for<N, 8>();
+  cplx64 x[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    x[r] = cplx64{0.0, 0.0};
+    if (!(ZP && (r == 3 || r == 4)) && active)
+      x[r] = TPP % sm_pad<cplx64>() == 0 ? buf[sm_at<cplx64>((unsigned)t) + sm_idx<cplx64>(r * TPP)]
+                                         : buf[sm_at<cplx64>((unsigned)(t + r * TPP))];
+  }
+  fx_fft_from<N, DIR, ZP, DP, REG>(x, buf, t, active, tw, scale2, out, out_scale);
 }
 
 // `t` in [0, N / VPT): the thread's index within its pencil's group.  ZP: the pencil is
@@ -819,11 +832,16 @@ struct RowPair {
   __device__ __forceinline__ static bool mirrored(int t, int r) { return N - t - r * TPP < NX; }
 };
 
-// Inverse transform of a row pair into the pencil `buf` (real part: row 0, imaginary part: row 1).
-// DP as in pencil_fft.
-template <int N, typename C, int VPT, bool DP, typename TW>
+// What a transform leaves in registers: fixed-point values and their scale in FP64 (a TwFx table).
+template <typename C, typename TW>
+using reg_of = typename std::conditional<std::is_same<TW, TwFx>::value, cfx, C>::type;
+
+// Inverse transform of a row pair (real part: row 0, imaginary part: row 1) into the pencil `buf`,
+// or (REG) into `out`: out[q] = element t + q TPP.  DP as in pencil_fft.
+template <int N, typename C, int VPT, bool DP, bool REG = false, typename TW>
 __device__ __forceinline__ void rows_inverse(C *buf, int t, bool active, RowPair<N, C, VPT> &x,
-                                             const TW *__restrict__ tw) {
+                                             const TW *__restrict__ tw, reg_of<C, TW> *out = nullptr,
+                                             FxScale *out_scale = nullptr) {
   using RP = RowPair<N, C, VPT>;
   constexpr int NI = RP::NI, TPP = RP::TPP;
   if constexpr (std::is_same<TW, TwFx>::value) {
@@ -869,7 +887,8 @@ __device__ __forceinline__ void rows_inverse(C *buf, int t, bool active, RowPair
       for (int r = 0; r < 8; ++r) fb[9u * (unsigned)t + r] = v[r];
     }
     group_sync<TPP>();
-    fx_stages<N, +1, 8, DP>(fb, t, active, tw, sc, sc.shift, 0);
+    fx_stages<N, +1, 8, DP, REG>(fb, t, active, tw, sc, sc.shift, 0, out);
+    if constexpr (REG) *out_scale = sc;
   } else {
     C v[VPT];
 #pragma unroll
@@ -896,27 +915,20 @@ __device__ __forceinline__ void rows_inverse(C *buf, int t, bool active, RowPair
       for (int r = 0; r < VPT; ++r) wp[sm_idx<C>(r)] = v[r];
     }
     group_sync<TPP>();
-    stockham_stages<N, +1, VPT, C, VPT, false>(buf, t, active, tw);
+    stockham_stages<N, +1, VPT, C, VPT, false, false, REG>(buf, t, active, tw, out);
   }
 }
 
-// Forward transform of the pencil `buf` and the half spectra of its two rows, doubled (the split's
-// factor 1/2 is left out; fixed point: scaled by 2^scale2), to dst and dst + NX.
-template <int N, typename C, int VPT, bool DP, typename TW, typename Post>
-__device__ __forceinline__ void rows_forward(C *buf, int t, bool active, C *__restrict__ dst,
-                                             const TW *__restrict__ tw, int scale2, Post post) {
+// The half spectra of the two rows of a forward-transformed pencil, from the values its last stage
+// left in registers: doubled (the split's factor 1/2 is left out; fixed point: scaled by 2^scale2),
+// through `post`, to dst and dst + NX.
+template <int N, typename C, int VPT, bool DP, typename E, typename Post>
+__device__ __forceinline__ void rows_split(E *z, const FxScale &sc, C *buf, int t, bool active, C *__restrict__ dst,
+                                           int scale2, Post post) {
   using RP = RowPair<N, C, VPT>;
   constexpr int NI = RP::NI, TPP = RP::TPP, NX = RP::NX;
-  constexpr bool kFx = std::is_same<TW, TwFx>::value;
-  using E = typename std::conditional<kFx, cfx, C>::type;
+  constexpr bool kFx = std::is_same<E, cfx>::value;
   E *eb = reinterpret_cast<E *>(buf);
-  E z[VPT];
-  FxScale sc{};
-  if constexpr (kFx) {
-    fx_pencil_fft<N, -1, false, DP, true>(buf, t, active, tw, 0, z, &sc);
-  } else {
-    stockham_stages<N, -1, 1, C, VPT, false, false, true>(buf, t, active, tw, z);
-  }
   // (the last stage has a barrier after its reads)
   if (active) {
 #pragma unroll
@@ -946,6 +958,39 @@ __device__ __forceinline__ void rows_forward(C *buf, int t, bool active, C *__re
       dst[NX + t + i * TPP] = y1;
     }
   }
+}
+
+// Forward transform of the pencil `buf` and the half spectra of its two rows (rows_split).
+template <int N, typename C, int VPT, bool DP, typename TW, typename Post>
+__device__ __forceinline__ void rows_forward(C *buf, int t, bool active, C *__restrict__ dst,
+                                             const TW *__restrict__ tw, int scale2, Post post) {
+  reg_of<C, TW> z[VPT];
+  FxScale sc{};
+  if constexpr (std::is_same<TW, TwFx>::value) fx_pencil_fft<N, -1, false, DP, true>(buf, t, active, tw, 0, z, &sc);
+  else stockham_stages<N, -1, 1, C, VPT, false, false, true>(buf, t, active, tw, z);
+  rows_split<N, C, VPT, DP>(z, sc, buf, t, active, dst, scale2, post);
+}
+
+// The same of the values x[r] = element t + r N/8 that the group's threads hold (radix 8).
+template <int N, typename C, bool DP, typename TW, typename Post>
+__device__ __forceinline__ void rows_forward_from(C *x, C *buf, int t, bool active, C *__restrict__ dst,
+                                                  const TW *__restrict__ tw, int scale2, Post post) {
+  constexpr int TPP = tpp_for<N, 8>();
+  reg_of<C, TW> z[8];
+  FxScale sc{};
+  if constexpr (std::is_same<TW, TwFx>::value) {
+    fx_fft_from<N, -1, false, DP, true>(x, buf, t, active, tw, 0, z, &sc);
+  } else {
+    if (active) {
+      dft8_first_fma<-1, false>(x);
+      C *wp = buf + sm_at<C>((unsigned)(t * 8));
+#pragma unroll
+      for (int r = 0; r < 8; ++r) wp[sm_idx<C>(r)] = x[r];
+    }
+    group_sync<TPP>();
+    stockham_stages<N, -1, 8, C, 8, false, false, true>(buf, t, active, tw, z);
+  }
+  rows_split<N, C, 8, DP>(z, sc, buf, t, active, dst, scale2, post);
 }
 
 // FFT index of kept index j (0..2K) along a truncated axis: j for j <= K, else j - (2K+1) + N.

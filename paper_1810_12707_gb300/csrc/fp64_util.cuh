@@ -1,0 +1,43 @@
+// fp64_util.cuh -- FP64 reciprocal, quotient and square root in few FP64 instructions, for kernels
+// that the FP64 pipe bounds (1.7 fused multiply-adds per clock and SM on GB300).  Each starts from the
+// hardware's approximation (relative error e of about 2^-20) and takes one step of Householder's
+// third-order iteration, whose remaining error, of order e^3, is below 2^-57: only the last fused
+// multiply-add rounds.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace mhd {
+
+// 1 / x = r (1 + e + e^2), e = 1 - x r: four instructions, about half a division's.  A NaN for x = 0
+// and x infinite.
+__device__ __forceinline__ double rcp3(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// Whether x is a normal, positive or negative, finite number whose reciprocal is one too.
+__device__ __forceinline__ bool rcp3_covers(double x) {
+  const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  return h - 0x00200000u < 0x7fa00000u;
+}
+// m / x with r = 1 / x from rcp3: the quotient m r corrected by its remainder (Markstein), which
+// rounds correctly but for rare cases.  Three instructions.
+__device__ __forceinline__ double quotient(double m, double x, double r) {
+  const double q = m * r;
+  return fma(fma(-x, q, m), r, q);
+}
+
+// sqrt(x) = s (1 + e/2 + 3 e^2 / 8), s = x y, e = 1 - s y, y the approximate 1 / sqrt(x): five
+// instructions; zero, subnormal, negative, infinite and NaN arguments take the library's root.
+__device__ __forceinline__ double sqrt3(double x) {
+  if ((unsigned)__double2hiint(x) - 0x00100000u >= 0x7fe00000u) return sqrt(x);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double s = x * y, e = fma(-s, y, 1.0);
+  return fma(s, e * fma(0.375, e, 0.5), s);
+}
+
+}  // namespace mhd

@@ -575,8 +575,8 @@ __global__ void step_dt_kernel(unsigned long long *__restrict__ smax_bits, const
   coef[inst] = c;
 }
 
-// One block: reduce the diagnostic partials of one instance in a fixed order and add the
-// spectral terms.  out: [0] ke [1] me [2] eint [3] cross_hel [4] mean_speed [5] mean_bmag
+// Reduce the diagnostic partials of one instance in a fixed order, a block per quantity, and add the
+// spectral terms (block 7).  out: [0] ke [1] me [2] eint [3] cross_hel [4] mean_speed [5] mean_bmag
 // [6] smax [7] mean_rho [8..10] mean_m [11..13] mean_b [14] divb_rms [15] t [16] dt_last
 // [17] step [18] status.
 __global__ void diag_finish_kernel(const double *__restrict__ part, int nparts, const double *__restrict__ dpart,
@@ -584,7 +584,8 @@ __global__ void diag_finish_kernel(const double *__restrict__ part, int nparts, 
                                    const TimeState *__restrict__ ts, double *__restrict__ out, int n, int K) {
   __shared__ double red[32];
   const double inv_n3 = 1.0 / ((double)n * n * n);
-  for (int q = 0; q < 7; ++q) {
+  if (blockIdx.x < 7) {
+    const int q = blockIdx.x;
     double v = 0.0;
     if (q < 6) {
       for (int i = threadIdx.x; i < nparts; i += blockDim.x) v += part[(size_t)i * 8 + q];
@@ -594,6 +595,7 @@ __global__ void diag_finish_kernel(const double *__restrict__ part, int nparts, 
       v = block_nan_max(v, red);
     }
     if (threadIdx.x == 0) out[q] = q < 6 ? v * inv_n3 : v;
+    return;
   }
   double d = 0.0;
   for (int i = threadIdx.x; i < ndparts; i += blockDim.x) d += dpart[i];
@@ -746,7 +748,7 @@ cudaError_t launch_diag_finish(const double *part, int nparts, const cplx64 *sta
   divb_partials_kernel<<<kDivbBlocks, 256, 0, s>>>(state, dpart, d.k);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  diag_finish_kernel<<<1, 1024, 0, s>>>(part, nparts, dpart, kDivbBlocks, state, phys, ts, out, d.n, d.k);
+  diag_finish_kernel<<<8, 1024, 0, s>>>(part, nparts, dpart, kDivbBlocks, state, phys, ts, out, d.n, d.k);
   return cudaGetLastError();
 }
 

@@ -15,6 +15,7 @@
 // real-space array ever reaches HBM), and their forward transforms leave as truncated half
 // spectra.  Rows are indexed r = z*N + y; a block owns PAIRS consecutive row pairs.
 #include "fft_device.cuh"
+#include "fp64_util.cuh"
 #include "launch_util.cuh"
 #include "tma_util.cuh"
 
@@ -69,17 +70,6 @@ constexpr int flux_min_blocks() {
 // 512^3 20.5 -> 19.8, but 256^3 2.31 -> 2.33).
 template <int N, typename C>
 constexpr bool flux_ahead() { return std::is_same<C, cplx64>::value ? N != 512 : !std::is_same<C, cdf>::value; }
-
-// 1 / x from the hardware's approximation r0 (relative error e, about 2^-20) by Householder's
-// iteration of third order, r0 (1 + e + e^2) with e = 1 - x r0: the neglected e^3 is below 2^-57, so
-// only the last fused multiply-add rounds.  Four FP64 instructions where the division takes about
-// twice as many.  Not finite for x = 0, infinite or NaN (a NaN).
-__device__ __forceinline__ double rcp3(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
 
 // |x| as an FP32 number from the high word alone, truncated (at most 2^-20 relative below |x|);
 // infinite from 2^128 on and for a NaN, 0 below 2^-126.  Integer instructions: a conversion costs
@@ -535,149 +525,145 @@ __device__ __forceinline__ void x_load(double v, dfr &r) { r = dfr_from_double(v
 __device__ __forceinline__ double x_store(double v) { return v; }
 __device__ __forceinline__ double x_store(dfr v) { return dfr_to_double(v); }
 
-template <int N, typename C, typename TW>
-// Rows from `row_begin` on (a multiple of 2 PAIRS); the real arrays hold rows from `row_begin`
-// with field stride `fstride` (N^3 for whole fields, less for a slab of z-planes).
-__global__ void __launch_bounds__(kMaxThreads) set_x_kernel(const double *__restrict__ rho, const double *__restrict__ u,
-                             const double *__restrict__ b, C *__restrict__ out, int K,
-                             const TW *__restrict__ tw, size_t row_begin, size_t fstride) {
-  using R = typename C::value_type;
-  constexpr int KT = (N - 1) / 3;  // the 2/3-rule cut-off, fixed by N
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C *sm = reinterpret_cast<C *>(smem_raw);
-  constexpr int P = pencil_pitch<C>(N);
-  constexpr int PAIRS = pairs_for(N);
-  constexpr size_t NN = (size_t)N * N;
-  constexpr int NX = KT + 1;
-  const size_t row0 = row_begin + (size_t)blockIdx.x * PAIRS * 2;
-  const int nthr = blockDim.x;
+// One group of N/8 threads per pencil (field f = id mod 7, row pair id / 7), kXThreads threads a block:
+// every thread's values of the two rows are the inputs of its first stage, and the last stage's
+// results go out from registers, so the fields' groups share nothing but the density rows (from L1)
+// and no block barrier.  One block of all 7 fields, the earlier form, left 5 of its 6 groups idle for
+// the seventh field at N = 512 and packed through shared memory: FP64 256^3 set 1.68 -> 0.50 ms, get
+// 1.75 -> 0.51 ms; IEEE set 2.92 -> 2.55 ms.
+constexpr int kXThreads = 256;
+template <int N>
+constexpr int x_groups() { return kXThreads / tpp_for<N, 8>(); }
 
-  for (int q = threadIdx.x; q < PAIRS * N; q += nthr) {
-    const int p = q / N, j = q - p * N;
-    const size_t i0 = (row0 - row_begin + 2 * p) * N + j, i1 = i0 + N;
-    const double r0 = rho[i0], r1 = rho[i1];
-    C *pen = sm + p * 7 * P + sm_idx<C>(j);
-    R a, c;
-    x_load(r0, a);
-    x_load(r1, c);
-    pen[0] = C{a, c};
+// The 7 real fields as three arrays (rho; 3 of one vector; 3 of the other) with field stride `stride`.
+template <typename T>
+struct Fields7 {
+  T *a, *b, *c;
+  size_t stride;
+  __device__ __forceinline__ T *field(int f) const {
+    return f == 0 ? a : f < 4 ? b + (f - 1) * stride : c + (f - 4) * stride;
+  }
+};
+
+// Rows from `row_begin` on (even); the real arrays hold rows from `row_begin` (field stride N^3 for
+// whole fields, less for a slab of z-planes).
+template <int N, typename C, typename TW>
+__global__ void __launch_bounds__(kXThreads) set_x_kernel(Fields7<const double> in, C *__restrict__ out,
+                                                          const TW *__restrict__ tw, size_t row_begin, int pencils) {
+  using R = typename C::value_type;
+  constexpr int NX = (N - 1) / 3 + 1, TPP = tpp_for<N, 8>(), P = pencil_pitch<C>(N);
+  constexpr size_t NN = (size_t)N * N;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int g = threadIdx.x / TPP, t = threadIdx.x - g * TPP;
+  const int id = blockIdx.x * x_groups<N>() + g;
+  const bool active = id < pencils;
+  const int f = active ? id % 7 : 0;
+  const size_t pair = active ? id / 7 : 0;
+
+  C x[8];
+  const double *src = in.field(f) + 2 * pair * N + t;
+  double v0[8], v1[8];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      x_load(r0 * u[d * fstride + i0], a);
-      x_load(r1 * u[d * fstride + i1], c);
-      pen[(1 + d) * P] = C{a, c};
-      x_load(b[d * fstride + i0], a);
-      x_load(b[d * fstride + i1], c);
-      pen[(4 + d) * P] = C{a, c};
+  for (int r = 0; r < 8; ++r) {
+    v0[r] = active ? src[r * TPP] : 0.0;
+    v1[r] = active ? src[N + r * TPP] : 0.0;
+  }
+  if (f >= 1 && f < 4) {  // m = rho u
+    const double *rho = in.a + 2 * pair * N + t;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      v0[r] = rho[r * TPP] * v0[r];
+      v1[r] = rho[N + r * TPP] * v1[r];
     }
   }
-  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    R a, b;
+    x_load(v0[r], a);
+    x_load(v1[r], b);
+    x[r] = C{a, b};
+  }
   // the split's factor 1/2: in fixed point a step of the results' exponents
   constexpr bool kFx = std::is_same<TW, TwFx>::value;
-  fft_pencils<N, -1, 8, kFx>(7 * PAIRS, [&](int id) { return sm + id * P; }, tw, kFx ? -1 : 0);
-  const auto half = [](C v) {
-    if constexpr (kFx) return v;
-    else return c_scale(v, (typename scale_of<C>::type)0.5);
-  };
-  for (int q = threadIdx.x; q < 7 * PAIRS * NX; q += nthr) {
-    const int k = q % NX;
-    const int r = q / NX;
-    const int f = r % 7, p = r / 7;
-    const C *pen = sm + (p * 7 + f) * P;
-    const C z = pen[sm_idx<C>(k)], zc = pen[sm_idx<C>((N - k) & (N - 1))];
-    C *dst = out + ((size_t)f * NN + row0 + 2 * p) * NX;
-    dst[k] = c_store(half(C{z.re + zc.re, z.im - zc.im}));
-    dst[NX + k] = c_store(half(C{z.im + zc.im, zc.re - z.re}));
-  }
+  rows_forward_from<N, C, kFx>(x, reinterpret_cast<C *>(smem_raw) + g * P, t, active,
+                               out + (f * NN + row_begin + 2 * pair) * NX, tw, -1,
+                               [](C v) { return c_store(c_scale(v, (typename scale_of<C>::type)0.5)); });
 }
 
 // ------------------------------------------------------------------------------------------
 // Inverse x transform to real rows
 // ------------------------------------------------------------------------------------------
+// Rows from `row_begin` on; `out` holds rows from `row_begin`; nf fields.  Pencils as in set_x_kernel.
 template <int N, typename C>
-// Rows from `row_begin` on; `out` holds rows from `row_begin` with field stride `fstride`.
-__global__ void __launch_bounds__(kMaxThreads) get_x_kernel(const C *__restrict__ in, double *__restrict__ out, int nf, int K,
-                             const typename tw_of<C>::type *__restrict__ tw, size_t row_begin, size_t fstride) {
-  constexpr int KT = (N - 1) / 3;  // the 2/3-rule cut-off, fixed by N
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C *sm = reinterpret_cast<C *>(smem_raw);
-  constexpr int P = pencil_pitch<C>(N);
-  constexpr int PAIRS = pairs_for(N);
+__global__ void __launch_bounds__(kXThreads) get_x_kernel(const C *__restrict__ in, Fields7<double> out, int nf,
+                                                          const typename tw_of<C>::type *__restrict__ tw,
+                                                          size_t row_begin, int pencils) {
+  constexpr int NX = (N - 1) / 3 + 1, TPP = tpp_for<N, 8>(), P = pencil_pitch<C>(N);
   constexpr size_t NN = (size_t)N * N;
-  constexpr int NX = KT + 1;
-  const size_t row0 = row_begin + (size_t)blockIdx.x * PAIRS * 2;
-  const int nthr = blockDim.x;
-
-  for (int q = threadIdx.x; q < nf * PAIRS * NX; q += nthr) {
-    const int k = q % NX;
-    const int r = q / NX;
-    const int f = r % nf, p = r / nf;
-    const C *src = in + ((size_t)f * NN + row0 + 2 * p) * NX;
-    C *pen = sm + (p * nf + f) * P;
-    const C x0 = src[k], x1 = src[NX + k];
-    if (k == 0) {
-      pen[0] = C{x0.re, x1.re};
-    } else {
-      pen[sm_idx<C>(k)] = C{x0.re - x1.im, x0.im + x1.re};
-      pen[sm_idx<C>(N - k)] = C{x0.re + x1.im, x1.re - x0.im};
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int g = threadIdx.x / TPP, t = threadIdx.x - g * TPP;
+  const int id = blockIdx.x * x_groups<N>() + g;
+  const bool active = id < pencils;
+  const int f = active ? id % nf : 0;
+  const size_t pair = active ? id / nf : 0;
+  RowPair<N, C, 8> x;
+  x.load(in + (f * NN + row_begin + 2 * pair) * NX, t, active);
+  reg_of<C, typename tw_of<C>::type> z[8];
+  FxScale sc{};
+  rows_inverse<N, C, 8, true, true>(reinterpret_cast<C *>(smem_raw) + g * P, t, active, x, tw, z, &sc);
+  if (active) {
+    double *dst = out.field(f) + 2 * pair * N + t;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      double v0, v1;
+      if constexpr (std::is_same<C, cplx64>::value) {
+        const uint32_t be = sc.ek + (uint32_t)sc.shift + 1u;
+        v0 = fx_to_double_dp(z[r].re, be);
+        v1 = fx_to_double_dp(z[r].im, be);
+        if (sc.bad) v0 = v1 = fx_double(0x7ff80000u, 0u);
+      } else {
+        v0 = x_store(z[r].re);
+        v1 = x_store(z[r].im);
+      }
+      dst[r * TPP] = v0;
+      dst[N + r * TPP] = v1;
     }
-  }
-  constexpr int NZ = pencil_zero_count<N>();
-  for (unsigned q = threadIdx.x; q < (unsigned)(nf * PAIRS * NZ); q += nthr) {
-    const unsigned z = q % NZ, r = q / NZ;
-    sm[r * P + sm_at<C>(pencil_zero<N>(z))] = C{0, 0};
-  }
-  __syncthreads();
-  fft_pencils<N, +1, 8, std::is_same<C, cplx64>::value>(nf * PAIRS, [&](int id) { return sm + id * P; }, tw);
-  for (int q = threadIdx.x; q < nf * PAIRS * N; q += nthr) {
-    const int j = q % N;
-    const int r = q / N;
-    const int f = r % nf, p = r / nf;
-    const C z = sm[(p * nf + f) * P + sm_idx<C>(j)];
-    const size_t i0 = f * fstride + (row0 - row_begin + 2 * p) * N + j;
-    out[i0] = x_store(z.re);
-    out[i0 + N] = x_store(z.im);
   }
 }
 
 // ------------------------------------------------------------------------------------------
 // Inverse x transform of the state with grid diagnostics
 // ------------------------------------------------------------------------------------------
+// A block owns PAIRS row pairs and one group per pencil (7 PAIRS of them) where 448 threads hold them.
+// The sums' constant factors are applied once per thread.  Bound by the FP64 pipe: per point one
+// reciprocal, three corrected quotients, three roots, a logarithm and about 20 more instructions
+// (fp64_util.cuh; 256^3 7.15 -> 3.84 ms against divisions, library roots and 7 pencils on 6 groups).
+constexpr int kDiagThreads = 448;
 template <int N>
-__global__ void __launch_bounds__(kMaxThreads) diag_x_kernel(const cplx64 *__restrict__ in, const PhysDev *__restrict__ phys,
-                              double *__restrict__ part, int K, const TwFx *__restrict__ tw) {
-  constexpr int KT = (N - 1) / 3;  // the 2/3-rule cut-off, fixed by N
+__global__ void __launch_bounds__(kDiagThreads) diag_x_kernel(const cplx64 *__restrict__ in,
+                                                              const PhysDev *__restrict__ phys,
+                                                              double *__restrict__ part,
+                                                              const TwFx *__restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx64 *sm = reinterpret_cast<cplx64 *>(smem_raw);
   __shared__ double red[32];
-  constexpr int P = pencil_pitch<cplx64>(N);
+  constexpr int P = pencil_pitch<cplx64>(N), TPP = tpp_for<N, 8>();
   constexpr int PAIRS = pairs_for(N);
   constexpr size_t NN = (size_t)N * N;
-  constexpr int NX = KT + 1;
+  constexpr int NX = (N - 1) / 3 + 1;
   const size_t row0 = (size_t)blockIdx.x * PAIRS * 2;
   const int nthr = blockDim.x;
 
-  for (int q = threadIdx.x; q < 7 * PAIRS * NX; q += nthr) {
-    const int k = q % NX;
-    const int r = q / NX;
-    const int f = r % 7, p = r / 7;
-    const cplx64 *src = in + ((size_t)f * NN + row0 + 2 * p) * NX;
-    cplx64 *pen = sm + (p * 7 + f) * P;
-    const cplx64 x0 = src[k], x1 = src[NX + k];
-    if (k == 0) {
-      pen[0] = cplx64{x0.re, x1.re};
-    } else {
-      pen[sm_idx<cplx64>(k)] = cplx64{x0.re - x1.im, x0.im + x1.re};
-      pen[sm_idx<cplx64>(N - k)] = cplx64{x0.re + x1.im, x1.re - x0.im};
-    }
-  }
-  constexpr int NZ = pencil_zero_count<N>();
-  for (unsigned q = threadIdx.x; q < (unsigned)(7 * PAIRS * NZ); q += nthr) {
-    const unsigned z = q % NZ, r = q / NZ;
-    sm[r * P + sm_at<cplx64>(pencil_zero<N>(z))] = cplx64{0.0, 0.0};
+  const int g = threadIdx.x / TPP, t = threadIdx.x - g * TPP, G = nthr / TPP;
+  for (int base = 0; base < 7 * PAIRS; base += G) {
+    const int id = base + g;
+    const bool active = g < G && id < 7 * PAIRS;
+    const int f = active ? id % 7 : 0, p = active ? id / 7 : 0;
+    RowPair<N, cplx64, 8> x;
+    x.load(in + ((size_t)f * NN + row0 + 2 * p) * NX, t, active);
+    rows_inverse<N, cplx64, 8, false>(sm + (active ? id : 0) * P, t, active, x, tw);
   }
   __syncthreads();
-  fft_pencils<N, +1, 8>(7 * PAIRS, [&](int id) { return sm + id * P; }, tw);
 
   const double cs2 = phys[0].cs * phys[0].cs;
   double acc[6] = {0, 0, 0, 0, 0, 0};
@@ -695,19 +681,35 @@ __global__ void __launch_bounds__(kMaxThreads) diag_x_kernel(const cplx64 *__res
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const double rho = v[h][0];
-      const double ux = v[h][1] / rho, uy = v[h][2] / rho, uz = v[h][3] / rho;
       const double bx = v[h][4], by = v[h][5], bz = v[h][6];
-      const double u2 = ux * ux + uy * uy + uz * uz;
       const double b2 = bx * bx + by * by + bz * bz;
-      acc[0] += 0.5 * rho * u2;
-      acc[1] += 0.5 * b2;
-      acc[2] += cs2 * rho * log(rho);
-      acc[3] += ux * bx + uy * by + uz * bz;
-      acc[4] += sqrt(u2);
-      acc[5] += sqrt(b2);
-      smax = nan_max(smax, sqrt(u2) + sqrt(cs2 + b2 / rho));
+      double ux, uy, uz, c2;
+      if (rcp3_covers(rho)) {
+        const double ir = rcp3(rho);
+        ux = quotient(v[h][1], rho, ir);
+        uy = quotient(v[h][2], rho, ir);
+        uz = quotient(v[h][3], rho, ir);
+        c2 = fma(b2, ir, cs2);
+      } else {
+        ux = v[h][1] / rho;
+        uy = v[h][2] / rho;
+        uz = v[h][3] / rho;
+        c2 = cs2 + b2 / rho;
+      }
+      const double u2 = ux * ux + uy * uy + uz * uz;
+      const double su = sqrt3(u2);
+      acc[0] = fma(rho, u2, acc[0]);
+      acc[1] += b2;
+      acc[2] = fma(rho, log(rho), acc[2]);
+      acc[3] = fma(ux, bx, fma(uy, by, fma(uz, bz, acc[3])));
+      acc[4] += su;
+      acc[5] += sqrt3(b2);
+      smax = nan_max(smax, su + sqrt3(c2));
     }
   }
+  acc[0] *= 0.5;
+  acc[1] *= 0.5;
+  acc[2] *= cs2;
   for (int i = 0; i < 6; ++i) {
     const double s = block_sum(acc[i], red);
     if (threadIdx.x == 0) part[(size_t)blockIdx.x * 8 + i] = s;
@@ -781,34 +783,26 @@ cudaError_t flux_n(const C *in, C *out, const PhysDev *phys, unsigned long long 
 template <int N, typename C, typename TW>
 cudaError_t set_n(const double *rho, const double *u, const double *b, C *out, const Dims &d,
                   const TW *tw, cudaStream_t s, size_t row_begin, size_t nrows, size_t fstride) {
-  constexpr int PAIRS = pairs_for(N);
-  if (row_begin % (2 * PAIRS) || nrows % (2 * PAIRS)) return cudaErrorInvalidValue;
-  const int blocks = (int)(nrows / (2 * PAIRS));
-  if (blocks == 0) return cudaSuccess;
-  const int threads = threads_for(tpp_for<N, 8>(), 7 * PAIRS);
-  const size_t smem = (size_t)7 * PAIRS * pencil_pitch<C>(N) * sizeof(C);
-  if (smem > 48 * 1024) {
-    cudaError_t e = ensure_smem<set_x_kernel<N, C, TW>>((int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  set_x_kernel<N, C, TW><<<blocks, threads, smem, s>>>(rho, u, b, out, d.k, tw, row_begin, fstride);
+  if (row_begin % 2 || nrows % 2) return cudaErrorInvalidValue;
+  const long long pencils = 7LL * (long long)(nrows / 2);
+  if (pencils == 0) return cudaSuccess;
+  const unsigned blocks = (unsigned)((pencils + x_groups<N>() - 1) / x_groups<N>());
+  const size_t smem = (size_t)x_groups<N>() * pencil_pitch<C>(N) * sizeof(C);  // below 48 KB for every N
+  set_x_kernel<N, C, TW><<<blocks, kXThreads, smem, s>>>(Fields7<const double>{rho, u, b, fstride}, out, tw, row_begin,
+                                                         (int)pencils);
   return cudaGetLastError();
 }
 
 template <int N, typename C>
-cudaError_t get_n(const C *in, double *out, int nf, const Dims &d, const typename tw_of<C>::type *tw, cudaStream_t s,
-                  size_t row_begin, size_t nrows, size_t fstride) {
-  constexpr int PAIRS = pairs_for(N);
-  if (row_begin % (2 * PAIRS) || nrows % (2 * PAIRS)) return cudaErrorInvalidValue;
-  const int blocks = (int)(nrows / (2 * PAIRS));
-  if (blocks == 0) return cudaSuccess;
-  const int threads = threads_for(tpp_for<N, 8>(), nf * PAIRS);
-  const size_t smem = (size_t)nf * PAIRS * pencil_pitch<C>(N) * sizeof(C);
-  if (smem > 48 * 1024) {
-    cudaError_t e = ensure_smem<get_x_kernel<N, C>>((int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  get_x_kernel<N, C><<<blocks, threads, smem, s>>>(in, out, nf, d.k, tw, row_begin, fstride);
+cudaError_t get_n(const C *in, double *a, double *b, double *c, int nf, const Dims &d,
+                  const typename tw_of<C>::type *tw, cudaStream_t s, size_t row_begin, size_t nrows, size_t fstride) {
+  if (row_begin % 2 || nrows % 2 || nf < 1 || nf > 7) return cudaErrorInvalidValue;
+  const long long pencils = (long long)nf * (long long)(nrows / 2);
+  if (pencils == 0) return cudaSuccess;
+  const unsigned blocks = (unsigned)((pencils + x_groups<N>() - 1) / x_groups<N>());
+  const size_t smem = (size_t)x_groups<N>() * pencil_pitch<C>(N) * sizeof(C);
+  get_x_kernel<N, C><<<blocks, kXThreads, smem, s>>>(in, Fields7<double>{a, b, c, fstride}, nf, tw, row_begin,
+                                                     (int)pencils);
   return cudaGetLastError();
 }
 
@@ -817,13 +811,13 @@ cudaError_t diag_n(const cplx64 *in, const PhysDev *phys, double *part, const Di
                    const TwFx *tw, cudaStream_t s) {
   constexpr int PAIRS = pairs_for(N);
   const int blocks = N * N / (2 * PAIRS);
-  const int threads = threads_for(tpp_for<N, 8>(), 7 * PAIRS);
+  const int threads = threads_for(tpp_for<N, 8>(), 7 * PAIRS, kDiagThreads);
   const size_t smem = (size_t)7 * PAIRS * pencil_pitch<cplx64>(N) * sizeof(cplx64);
   if (smem > 48 * 1024) {
     cudaError_t e = ensure_smem<diag_x_kernel<N>>((int)smem);
     if (e != cudaSuccess) return e;
   }
-  diag_x_kernel<N><<<blocks, threads, smem, s>>>(in, phys, part, d.k, tw);
+  diag_x_kernel<N><<<blocks, threads, smem, s>>>(in, phys, part, tw);
   return cudaGetLastError();
 }
 
@@ -886,12 +880,25 @@ cudaError_t launch_set_x_rows(const double *rho, const double *u, const double *
 cudaError_t launch_get_x(const cplx64 *in, double *out, int nfields, const Dims &d,
                          const TwFx *tw, cudaStream_t s) {
   const size_t nn = (size_t)d.n * d.n;
-  MHD_DISPATCH_N(d.n, (get_n<N>(in, out, nfields, d, tw, s, 0, nn, nn * d.n)));
+  const size_t n3 = nn * d.n;
+  MHD_DISPATCH_N(d.n, (get_n<N>(in, out, out + n3, out + 4 * n3, nfields, d, tw, s, 0, nn, n3)));
+}
+
+cudaError_t launch_get_x(const cplx64 *in, double *a, double *b, double *c, const Dims &d, const TwFx *tw,
+                         cudaStream_t s) {
+  const size_t nn = (size_t)d.n * d.n;
+  MHD_DISPATCH_N(d.n, (get_n<N>(in, a, b, c, 7, d, tw, s, 0, nn, nn * d.n)));
+}
+
+cudaError_t launch_get_x(const cdf *in, double *a, double *b, double *c, const Dims &d, const cdf *tw,
+                         cudaStream_t s) {
+  const size_t nn = (size_t)d.n * d.n;
+  MHD_DISPATCH_N(d.n, (get_n<N>(in, a, b, c, 7, d, tw, s, 0, nn, nn * d.n)));
 }
 
 cudaError_t launch_get_x_rows(const cplx64 *in, double *out, int nfields, const Dims &d, const TwFx *tw,
                               cudaStream_t s, size_t row_begin, size_t nrows, size_t fstride) {
-  MHD_DISPATCH_N(d.n, (get_n<N>(in, out, nfields, d, tw, s, row_begin, nrows, fstride)));
+  MHD_DISPATCH_N(d.n, (get_n<N>(in, out, out + fstride, out + 4 * fstride, nfields, d, tw, s, row_begin, nrows, fstride)));
 }
 
 cudaError_t launch_set_x_rows(const double *rho, const double *u, const double *b, cdf *out, const Dims &d,
@@ -901,7 +908,7 @@ cudaError_t launch_set_x_rows(const double *rho, const double *u, const double *
 
 cudaError_t launch_get_x_rows(const cdf *in, double *out, int nfields, const Dims &d, const cdf *tw, cudaStream_t s,
                               size_t row_begin, size_t nrows, size_t fstride) {
-  MHD_DISPATCH_N(d.n, (get_n<N>(in, out, nfields, d, tw, s, row_begin, nrows, fstride)));
+  MHD_DISPATCH_N(d.n, (get_n<N>(in, out, out + fstride, out + 4 * fstride, nfields, d, tw, s, row_begin, nrows, fstride)));
 }
 
 cudaError_t launch_diag_x(const cplx64 *in, const PhysDev *phys, double *part, const Dims &d,

@@ -285,11 +285,11 @@ mhd_status state_fp64(mhd_ctx *c, int inst, const cplx64 **out) {
   return MHD_OK;
 }
 
-// inverse z then inverse y of 7 fields of one instance: S-layout `src` -> W2 [7][z][y][kx]
-mhd_status inverse_zy(mhd_ctx *c, const cplx64 *src) {
+// inverse z then inverse y of the first nf fields of one instance: S-layout `src` -> W2 [nf][z][y][kx]
+mhd_status inverse_zy(mhd_ctx *c, const cplx64 *src, int nf = 7) {
   const mhd::Dims &d = c->d;
-  CK(mhd::launch_col_inverse(src, c->W1, d.n, 7, d.nk * d.nx, c->tw, c->stream));
-  CK(mhd::launch_col_inverse(c->W1, c->W2, d.n, 7 * d.n, d.nx, c->tw, c->stream));
+  CK(mhd::launch_col_inverse(src, c->W1, d.n, nf, d.nk * d.nx, c->tw, c->stream));
+  CK(mhd::launch_col_inverse(c->W1, c->W2, d.n, nf * d.n, d.nx, c->tw, c->stream));
   return MHD_OK;
 }
 
@@ -298,18 +298,31 @@ mhd_status copy_out(mhd_ctx *c, void *dst, const void *src, size_t bytes, int on
   return MHD_OK;
 }
 
-// Inverse-transform 7 truncated spectra (S layout) of one instance into real rho/m/B outputs.
-mhd_status spectra_to_real(mhd_ctx *c, const cplx64 *src, double *a, double *b3, double *c3, int on_device) {
+// The inverse x pass of the 7 fields in W2 into rho/m/B outputs: straight into device arrays, through
+// W1 to the host.  Synchronises.
+template <typename C>
+mhd_status rows_out(mhd_ctx *c, const C *w2, const typename mhd::tw_of<C>::type *tw, double *a, double *b3, double *c3,
+                    int on_device) {
   const size_t n3 = (size_t)c->d.n * c->d.n * c->d.n;
-  mhd_status st = inverse_zy(c, src);
-  if (st) return st;
-  double *real = reinterpret_cast<double *>(c->W1);
-  CK(mhd::launch_get_x(c->W2, real, 7, one(c), c->tw, c->stream));
-  if ((st = copy_out(c, a, real, n3 * sizeof(double), on_device))) return st;
-  if ((st = copy_out(c, b3, real + n3, 3 * n3 * sizeof(double), on_device))) return st;
-  if ((st = copy_out(c, c3, real + 4 * n3, 3 * n3 * sizeof(double), on_device))) return st;
+  if (on_device) {
+    CK(mhd::launch_get_x(w2, a, b3, c3, one(c), tw, c->stream));
+  } else {
+    mhd_status st;
+    double *real = reinterpret_cast<double *>(c->W1);
+    CK(mhd::launch_get_x(w2, real, real + n3, real + 4 * n3, one(c), tw, c->stream));
+    if ((st = copy_out(c, a, real, n3 * sizeof(double), 0))) return st;
+    if ((st = copy_out(c, b3, real + n3, 3 * n3 * sizeof(double), 0))) return st;
+    if ((st = copy_out(c, c3, real + 4 * n3, 3 * n3 * sizeof(double), 0))) return st;
+  }
   CK(cudaStreamSynchronize(c->stream));
   return MHD_OK;
+}
+
+// Inverse-transform 7 truncated spectra (S layout) of one instance into real rho/m/B outputs.
+mhd_status spectra_to_real(mhd_ctx *c, const cplx64 *src, double *a, double *b3, double *c3, int on_device) {
+  mhd_status st = inverse_zy(c, src);
+  if (st) return st;
+  return rows_out(c, c->W2, c->tw, a, b3, c3, on_device);
 }
 
 }  // namespace
@@ -733,17 +746,10 @@ mhd_status mhd_get_state(mhd_ctx *c, int32_t inst, double *rho, double *m, doubl
     const cdf *Sd = statedf(c, inst);
     if (!on_device && (st = get_state_host(c, Sd, c->twdf, rho, m, b)) != MHD_EINVAL) return st;
     const mhd::Dims &d = c->d;
-    const size_t n3 = (size_t)d.n * d.n * d.n;
     cdf *w1 = reinterpret_cast<cdf *>(c->W1), *w2 = reinterpret_cast<cdf *>(c->W2);
     CK(mhd::launch_col_inverse(Sd, w1, d.n, 7, d.nk * d.nx, c->twdf, c->stream));
     CK(mhd::launch_col_inverse(w1, w2, d.n, 7 * d.n, d.nx, c->twdf, c->stream));
-    double *real = reinterpret_cast<double *>(c->W1);
-    CK(mhd::launch_get_x_rows(w2, real, 7, one(c), c->twdf, c->stream, 0, (size_t)d.n * d.n, n3));
-    if ((st = copy_out(c, rho, real, n3 * sizeof(double), on_device))) return st;
-    if ((st = copy_out(c, m, real + n3, 3 * n3 * sizeof(double), on_device))) return st;
-    if ((st = copy_out(c, b, real + 4 * n3, 3 * n3 * sizeof(double), on_device))) return st;
-    CK(cudaStreamSynchronize(c->stream));
-    return MHD_OK;
+    return rows_out(c, w2, c->twdf, rho, m, b, on_device);
   }
   const cplx64 *src = nullptr;
   if ((st = state_fp64(c, inst, &src))) return st;
@@ -996,14 +1002,7 @@ mhd_status mhd_rhs(mhd_ctx *c, int32_t inst, double *drho, double *dm, double *d
   // W2 holds the RHS spectra; inverse_zy reads its source before overwriting W2
   CK(mhd::launch_col_inverse(c->W2, c->W1, d.n, 7, d.nk * d.nx, c->tw, c->stream));
   CK(mhd::launch_col_inverse(c->W1, c->W2, d.n, 7 * d.n, d.nx, c->tw, c->stream));
-  const size_t n3 = (size_t)d.n * d.n * d.n;
-  double *real = reinterpret_cast<double *>(c->W1);
-  CK(mhd::launch_get_x(c->W2, real, 7, d, c->tw, c->stream));
-  if ((st = copy_out(c, drho, real, n3 * sizeof(double), on_device))) return st;
-  if ((st = copy_out(c, dm, real + n3, 3 * n3 * sizeof(double), on_device))) return st;
-  if ((st = copy_out(c, db, real + 4 * n3, 3 * n3 * sizeof(double), on_device))) return st;
-  CK(cudaStreamSynchronize(c->stream));
-  return MHD_OK;
+  return rows_out(c, c->W2, c->tw, drho, dm, db, on_device);
 }
 
 }  // extern "C"
@@ -1357,7 +1356,7 @@ mhd_status mhd_spectra(mhd_ctx *c, int32_t inst, double *ek, double *em, int32_t
   const cplx64 *Si = nullptr;
   if ((st = state_fp64(c, inst, &Si))) return st;
   // u_hat: inverse z, y of the state; u = m / rho with the x passes; forward y, z
-  if ((st = inverse_zy(c, Si))) return st;
+  if ((st = inverse_zy(c, Si, 4))) return st;  // rho and m
   CK(mhd::launch_velocity_x(c->W2, c->W1, d, c->tw, c->stream));
   CK(mhd::launch_col_forward(c->W1, c->W2, d.n, 3 * d.n, d.nx, 1.0, c->tw, c->stream));
   CK(mhd::launch_col_forward(c->W2, c->W1, d.n, 3, d.nk * d.nx, 1.0 / (double)n3, c->tw, c->stream));
@@ -1365,8 +1364,10 @@ mhd_status mhd_spectra(mhd_ctx *c, int32_t inst, double *ek, double *em, int32_t
   // (clear of u_hat, 3 spec values, and of all that the du_x/dx chain below writes into W1: its
   // z-pass output and n^3 real values; W1 holds at least 7 n^3 doubles)
   cplx64 *gh = c->W1 + n3;
-  CK(mhd::launch_shells(c->W1, Si + 4 * d.spec, c->W2, gh, c->part, d, c->stream));
-  std::vector<double> sh((size_t)5 * ns);
+  // blocks per shell: as many as the partials' buffer holds sums of, at most 32
+  const int chunks = (int)std::min<size_t>(32, part_len / ((size_t)5 * ns));
+  CK(mhd::launch_shells(c->W1, Si + 4 * d.spec, c->W2, gh, c->part, d, chunks, c->stream));
+  std::vector<double> sh((size_t)5 * ns * chunks);
   CK(cudaMemcpyAsync(sh.data(), c->part, sh.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   // du_x/dx on the grid, then its moments
@@ -1387,6 +1388,8 @@ mhd_status mhd_spectra(mhd_ctx *c, int32_t inst, double *ek, double *em, int32_t
   CK(cudaMemcpyAsync(ap.data(), c->part, ap.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   double th = 0.0, m2 = 0.0, m3 = 0.0, hk = 0.0, hm = 0.0, dmax = 0.0;
+  for (size_t i = 0; i < (size_t)5 * ns; ++i)
+    for (int q = 1; q < chunks; ++q) sh[i] += sh[(size_t)q * 5 * ns + i];
   for (int s = 0; s < ns; ++s) {
     if (ek) ek[s] = sh[5 * s];
     if (em) em[s] = sh[5 * s + 1];
