@@ -53,6 +53,21 @@ struct KeptRows {
   }
 };
 
+// Distance between a tile's pencils.  The tile's loads and stores go through shared memory with a
+// row's tc columns in consecutive lanes, so the L = 128 / element size lanes of one wavefront cover
+// max(1, L / tc) consecutive elements of min(tc, L) pencils: a pitch of L / tc modulo L puts them on
+// distinct banks (1 for tc >= L).  With the odd pitch of the x passes every access of the tiles
+// narrower than L had two-way conflicts: 28 % of the wavefronts of the 256^3 mixed passes.  Groups of
+// less than L threads (the smallest grids) keep the odd pitch, their stages have several pencils in a
+// wavefront.
+template <int N, int TPP, typename CC>
+__host__ __device__ __forceinline__ int tile_pitch(int tc) {
+  constexpr int L = sm_pad<CC>(), base = sm_idx<CC>(N);
+  if constexpr (TPP < L) return base | 1;
+  const int want = tc >= L ? 1 : L / tc;  // modulo L
+  return base + (want + L - base % L) % L;
+}
+
 // CI, CO: element types in and out; CC: type of the transform arithmetic (= the output's).
 // A block has TC = 2^tsh columns and TC * N/VPT threads: thread (l0, c) = (tid >> tsh, tid & (TC-1))
 // moves rows l0, l0 + N/VPT, ... of column c, so consecutive threads touch consecutive columns of a
@@ -64,7 +79,7 @@ __device__ __forceinline__ void col_fft_tile(const CI *__restrict__ in, CO *__re
                                              int tsh, int cols, typename scale_of<CC>::type scale,
                                              const TW *__restrict__ tw, CC *sm) {
   constexpr int TPP = tpp_for<N, VPT>();
-  constexpr int P = pencil_pitch<CC>(N);
+  const int P = tile_pitch<N, TPP, CC>(1 << tsh);
   constexpr int K = (N - 1) / 3;  // the 2/3-rule cut-off, fixed by N
   constexpr int NK = 2 * K + 1;
   constexpr int LIN = DIR > 0 ? NK : N;
@@ -265,7 +280,7 @@ cudaError_t launch_col_v(const CI *in, CO *out, int nslab, int cols, double scal
   const int tsh = floor_log2(tc);  // a requested width that is not a power of two is rounded down
   tc = 1 << tsh;
   const int ntiles = (cols + tc - 1) / tc;
-  const size_t smem = (size_t)tc * pencil_pitch<CO>(N) * sizeof(CO) + tws_bytes<CO, N>();
+  const size_t smem = (size_t)tc * tile_pitch<N, TPP, CO>(tc) * sizeof(CO) + tws_bytes<CO, N>();
   const long long blocks = (long long)nslab * ntiles;
   if (blocks <= 0) return cudaSuccess;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
