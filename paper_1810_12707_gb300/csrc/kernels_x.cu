@@ -38,13 +38,14 @@ constexpr int threads_for(int tpp, int pencils, int max_threads = kMaxThreads) {
   return (t + 31) / 32 * 32;
 }
 
-// Block size of the flux pass.  At N = 256 and 512 several smaller blocks per SM let one block
-// transform while another waits at a barrier (measured on GB300 over 96..384 threads: 128 best at
-// 256^3 in both precisions, 192 at 512^3); below, the pencil count caps the block at 192 threads.
-// The 16-byte passes at 512^3 take 256 (two blocks of 128 registers a thread per SM): double-float
-// 4 % faster than 192, FP64 27.0 -> 22.8 ms.
-constexpr int flux_max_threads(int n, bool wide = false) {
-  return n == 256 ? 128 : n == 512 ? (wide ? 256 : 192) : kMaxThreads;
+// Block size of the flux pass: where one row pair fills a block (N >= 128), 4 groups, which take the 7
+// and 12 pencils in 2 + 3 rounds with one group idle in one of them (12 groups left 5 idle for the
+// fields, 8 left 4 idle for the last products).  128^3 double-float 0.303 -> 0.210 ms against 192
+// threads, 256^3 mixed 0.408 -> 0.346 against 128, 512^3 mixed 4.45 -> 4.41 against 192.  Below, where
+// few blocks have to hide each other's latency, one group per product (at most 192 threads): 64 threads
+// measured 0.059 against 0.049 ms for one 64^3 FP64 instance.
+constexpr int flux_max_threads(int n, int tpp) {
+  return n < 128 || n > 512 ? kMaxThreads : 4 * tpp;
 }
 // Values per thread of the flux pass's transforms: FP32 at N <= 256 uses radix 16 (measured
 // faster at 64^3 and 256^3); larger FP32 grids and FP64 use radix 8.
@@ -53,7 +54,7 @@ constexpr int flux_vpt() { return sizeof(C) == 8 && N <= 256 ? 16 : 8; }
 template <int N, typename C>
 constexpr int flux_threads() {
   return threads_for(tpp_for<N, flux_vpt<N, C>()>(), 12 * pairs_for(N),
-                     flux_max_threads(N, sizeof(C) == 16));
+                     flux_max_threads(N, tpp_for<N, flux_vpt<N, C>()>()));
 }
 // Blocks per SM the register allocation is sized for: about 170 registers a thread in FP64, 85 in
 // FP32 with radix 8 and 128 with radix 16 (its 16 values per thread).
