@@ -472,10 +472,17 @@ struct SlabPlan {
   double *slot[8];  // 7 fields x dz N^2 doubles each
 };
 
+// Up to this size a state crosses the host link in one piece (three launches and three copies): 8 slabs
+// of up to 8 launches, 7 copies and 4 event calls cost 0.5 to 0.9 ms of host time, more than the
+// overlap gains.  One piece against slabs, us: 32^3 set from pinned memory 63 / 459, get into fresh
+// pageable memory 71 / 952; 64^3 135 / 475, 159 / 1039; 128^3 759 / 868, 6425 / 40569.
+constexpr int kHostPieceMaxN = 128;
+
 // As many slots of N/8 z-planes as W1 holds behind the y-pass output, up to one per slab (so
 // that a transfer in can run ahead of the transforms); thinner slabs when not even two fit.
 bool slab_plan(mhd_ctx *c, SlabPlan *pl) {
   const mhd::Dims &d = c->d;
+  if (d.n <= kHostPieceMaxN) return false;
   const size_t n = d.n, nn = n * n;
   const size_t head = (7 * n * d.nk * d.nx + 15) / 16 * 16;  // y-pass output, complex values
   if (head >= c->w1_len) return false;
@@ -579,6 +586,7 @@ mhd_status async_staging(mhd_ctx *c, Staging *sg) {
   if (!c->oslots) {
     const size_t cap = footprint(c->d, c->precision) / 2;
     int dz = (int)(n / 8), ns = 8;
+    if ((int)n <= kHostPieceMaxN) dz = (int)n, ns = 1;  // one slab
     while (ns > 2 && (size_t)7 * ns * dz * nn * sizeof(double) > cap) --ns;
     while (dz > 1 && (size_t)7 * ns * dz * nn * sizeof(double) > cap) dz /= 2;
     const size_t bytes = (size_t)7 * ns * dz * nn * sizeof(double);
@@ -617,9 +625,11 @@ mhd_status get_state_staged(mhd_ctx *c, const C *src, const typename mhd::tw_of<
     double *slot = sg.slot[k];
     const size_t off = (size_t)z0 * nn, cnt = (size_t)dzc * nn;
     if (i >= sg.ns) e = cudaStreamWaitEvent(c->stream, sg.free[k], 0);  // slot copied out
-    for (int f = 0; f < 7 && e == cudaSuccess; ++f) {
-      const size_t slab0 = (size_t)f * n + z0;  // y pass of these z-planes
-      e = mhd::launch_col_inverse(w1 + slab0 * d.nk * d.nx, w2 + slab0 * n * d.nx, n, dzc, d.nx, tw, c->stream);
+    // y pass of these z-planes, field by field; all of them in one launch
+    const int ny = dzc == n ? 1 : 7, cnt_y = dzc == n ? 7 * n : dzc;
+    for (int f = 0; f < ny && e == cudaSuccess; ++f) {
+      const size_t slab0 = (size_t)f * n + z0;
+      e = mhd::launch_col_inverse(w1 + slab0 * d.nk * d.nx, w2 + slab0 * n * d.nx, n, cnt_y, d.nx, tw, c->stream);
     }
     if (e == cudaSuccess)
       e = mhd::launch_get_x_rows(w2, slot, 7, d1, tw, c->stream, (size_t)z0 * n, (size_t)dzc * n, cnt);
