@@ -56,7 +56,6 @@ PAPER_512_P100 = 512 ** 3 / 80.97
 
 def paper_baseline(n: int):
     return {256: PAPER_256_V100, 512: PAPER_512_P100}.get(n)
-FP64_PEAK_TFLOPS = 1.26   # 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz (nominal 1.25 TFLOP/s)
 FP32_PEAK_TFLOPS = 80.5   # 152 SMs x 128 FP32 FMA/clk x 2 flop x 2.07 GHz
 FP32_PEAK_TOPS = 40.27    # FP32 lane operations per second: 152 SMs x 128 lanes x 2.07 GHz (x 1e12)
 ORACLE_MAX_N = 256        # largest grid the oracle is timed on (about 16 GB of host memory)
@@ -136,6 +135,11 @@ def kernel_model(n: int, batch: int = 1, precision: str = "fp64"):
         # lane operations the double-float method performs (dfloat_ops)
         ops = dfloat_ops(n)
         m = {key: (b, ops[key]) for key, (b, f) in m.items()}
+    elif precision == "fp64":
+        # the FP64 passes transform in 64-bit fixed point: "flops" become the instructions per lane
+        # that the method needs (fixed_ops)
+        ops = fixed_ops(n)
+        m = {key: (b, ops[key]) for key, (b, f) in m.items()}
     return {key: (b * batch, f * batch) for key, (b, f) in m.items()}
 
 
@@ -183,13 +187,53 @@ def dfloat_ops(n: int) -> dict:
     }
 
 
+def fixed_fft_ops(n: int) -> float:
+    """Instructions per lane of one length-n complex transform of FP64 data in 64-bit fixed point:
+    the stages of dfloat_fft_ops with a complex sum 4 (two 32-bit halves of two parts), a complex
+    twiddle product 38 (12 multiplications of 32 x 32 bits, 26 splits, shifts and sums), a product by
+    sqrt(2)/2 10; and per value the conversion in 40 (exponent, size and shifts of two parts) and out
+    6 (two additions of the FP64 pipe and one integer instruction a part)."""
+    stages, rem = 0, n
+    while rem >= 8:
+        rem //= 8
+        stages += 1
+    dft8 = 26 * 4.0 + 4 * 10
+    ops = (n / 8) * dft8 + (stages - 1) * (n / 8) * (dft8 + 7 * 38)
+    if rem == 4:
+        ops += (n / 4) * (8 * 4 + 3 * 38)
+    elif rem == 2:
+        ops += (n / 2) * (2 * 4 + 38)
+    return ops + n * 46.0
+
+
+def fixed_ops(n: int) -> dict:
+    """Instructions per lane and launch of each FP64 kernel (one instance): transforms
+    (fixed_fft_ops), the grid products (about 30 FP64 and 40 other instructions per grid value) and the
+    spectral assembly with the update (about 90 FP64 and 60 others per mode).  An FP64 instruction
+    takes 75 of these slots' time on its own pipe; the figure counts it once."""
+    k = (n - 1) // 3
+    nx, nk = k + 1, 2 * k + 1
+    spec = nk * nk * nx
+    f = fixed_fft_ops(n)
+    return {
+        "inverse_z": 7 * nk * nx * f,
+        "inverse_y": 7 * n * nx * f,
+        "flux_x": (n * n / 2) * (19 * f + 2 * n * 70.0),
+        "step_dt": 0.0,
+        "forward_y": 12 * n * nx * f,
+        "forward_z": 12 * nk * nx * f,
+        "assemble_ab2": 150.0 * spec,
+        "assemble_iz": 150.0 * spec + 7 * nk * nx * f,
+    }
+
+
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch, from one ncu capture
 # per entry (summarised under profiles/).  A figure stands only while the sources that build the
 # kernel are the ones it was taken on: the entry keeps a hash of those files and is dropped
 # (traffic reported as null) as soon as they change.
 KERNEL_SOURCES = {
-    "flux_x": ("kernels_x.cu", "fft_device.cuh"),
-    "col": ("kernels_col.cu", "fft_device.cuh"),
+    "flux_x": ("kernels_x.cu", "fft_device.cuh", "fixed64.cuh"),
+    "col": ("kernels_col.cu", "fft_device.cuh", "fixed64.cuh"),
 }
 TRAFFIC = {
     # (kernel, n, batch, precision): (bytes per launch, source hash, capture)
@@ -505,7 +549,7 @@ def run_ours(args, name, cfg):
     # roofline of the dominant kernel (largest share of device time)
     hbm, hbm_src = peaks()
     model = kernel_model(n, batch, cfg["precision"])
-    alu_peak = {"fp64": FP64_PEAK_TFLOPS, "fp64df": FP32_PEAK_TOPS}.get(cfg["precision"], FP32_PEAK_TFLOPS)
+    alu_peak = {"fp64": FP32_PEAK_TOPS, "fp64df": FP32_PEAK_TOPS}.get(cfg["precision"], FP32_PEAK_TFLOPS)
     total_ms = sum(v[0] for v in prof.values())
     per = {}
     for kname, (tot, cnt) in prof.items():
@@ -526,7 +570,8 @@ def run_ours(args, name, cfg):
             unit, src = ("T FP32-ops/s", "FP32 lanes x clock: 152 SMs x 128 x 2.07 GHz (one operation per lane "
                          "per clock; the algorithmic count is the double-float method's FP32 operations)")
         elif prec == mhd.MHD_FP64:
-            unit, src = "TFLOP/s", "FP64 FMA units x clock (nominal 1.25 TFLOP/s; probe 1.19)"
+            unit, src = ("T instructions/s", "issue slots x lanes x clock: 152 SMs x 128 x 2.07 GHz (the count is the "
+                         "fixed-point method's instructions per lane)")
         else:
             unit, src = "TFLOP/s", "FP32 FMA units x clock (probe 74.4 TFLOP/s)"
         roof = {"bound": "alu", "achieved": per[top]["tflops"], "peak": alu_peak, "unit": unit,

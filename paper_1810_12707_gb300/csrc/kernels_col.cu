@@ -3,8 +3,8 @@
 // The data of one pass is viewed as [nslab][L][C]: the transform runs along L for each of the
 // nslab * C columns; the C columns of a slab are contiguous in memory.  A block takes TC
 // consecutive columns of one slab, so every row of the tile is one coalesced segment of TC complex
-// values.  The tile is transposed into shared memory as TC pencils of length N (pitch N + 1, which
-// spreads consecutive pencils over the banks), transformed by TC groups of N/VPT threads, and
+// values.  The tile is transposed into shared memory as TC pencils of length N (tile_pitch apart,
+// which spreads consecutive pencils over the banks), transformed by TC groups of N/VPT threads, and
 // written back.
 //   inverse (DIR = +1): L = 2K + 1 kept rows in, scattered to their FFT indices with the rest of
 //                       the pencil zero (the 2/3-rule truncation), all N rows out;
@@ -156,6 +156,7 @@ template <int N, int DIR, typename CI, typename CO, typename CC, int VPT, typena
 __global__ void col_fft_kernel(const CI *__restrict__ in, CO *__restrict__ out, int ntiles, int tsh,
                                int cols, typename scale_of<CC>::type scale, const TW *__restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   col_fft_tile<N, DIR, CI, CO, CC, VPT, TW>(in, out, blockIdx.x, ntiles, tsh, cols, scale, tw,
                                         reinterpret_cast<CC *>(smem_raw));
 }
@@ -170,6 +171,7 @@ __global__ void __launch_bounds__(256, 4) col_fft_kernel_b4(const CI *__restrict
                                                            typename scale_of<CC>::type scale,
                                                            const TW *__restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   col_fft_tile<N, DIR, CI, CO, CC, VPT, TW>(in, out, blockIdx.x, ntiles, tsh, cols, scale, tw,
                                         reinterpret_cast<CC *>(smem_raw));
 }
@@ -177,7 +179,8 @@ __global__ void __launch_bounds__(256, 4) col_fft_kernel_b4(const CI *__restrict
 // The kernel a pass launches.
 template <int N, int DIR, typename CI, typename CO, int VPT, typename TW = typename tw_of<CO>::type>
 constexpr auto col_kernel() {
-  if constexpr ((std::is_same<CO, cdf>::value && DIR < 0) || std::is_same<TW, TwFx>::value) return col_fft_kernel_b4<N, DIR, CI, CO, CO, VPT, TW>;
+  if constexpr ((std::is_same<CO, cdf>::value && DIR < 0) || std::is_same<TW, TwFx>::value)
+    return col_fft_kernel_b4<N, DIR, CI, CO, CO, VPT, TW>;
   else return col_fft_kernel<N, DIR, CI, CO, CO, VPT, TW>;
 }
 
@@ -300,9 +303,8 @@ cudaError_t launch_col_v(const CI *in, CO *out, int nslab, int cols, double scal
     cudaError_t e = ensure_smem<col_kernel<N, DIR, CI, CO, VPT, TW>()>((int)smem);
     if (e != cudaSuccess) return e;
   }
-  col_kernel<N, DIR, CI, CO, VPT, TW>()<<<(unsigned)blocks, tc * TPP, smem, s>>>(
-      in, out, ntiles, tsh, cols, (typename scale_of<CO>::type)scale, tw);
-  return cudaGetLastError();
+  return launch_after(col_kernel<N, DIR, CI, CO, VPT, TW>(), dim3((unsigned)blocks), dim3(tc * TPP), smem, s, in, out,
+                      ntiles, tsh, cols, (typename scale_of<CO>::type)scale, tw);
 }
 
 // Radix of a column pass: `vpt` 8 or 16 (FP32 only); 0 picks the library default (radix 8, and

@@ -214,6 +214,7 @@ __global__ void assemble_kernel(const FC *__restrict__ flux, const cplx64 *y_in,
                                 const cplx64 *__restrict__ force, int op_, int stage, int K, int batch,
                                 double inv_n3, FastDiv nx, FastDiv nk) {
   extern __shared__ double waves[];  // k_j, then k_j inv_n3, j < NK
+  after_previous();
   const int op = AB2 ? (int)ASM_AB2 : op_;
   const int NK = (int)nk.d;
   for (int j = threadIdx.x; j < NK; j += blockDim.x) {
@@ -367,6 +368,7 @@ __global__ void __launch_bounds__(256) assemble_df_kernel(
     const StepCoef *__restrict__ coef, const cplx32 *__restrict__ force, int op_, int stage, int K, int batch,
     float inv_n3, FastDiv nx, FastDiv nk) {
   const int op = AB2 ? (int)ASM_AB2 : op_;
+  after_previous();
   const unsigned spec = nk.d * nk.d * nx.d;
   for (int inst = blockIdx.y; inst < batch; inst += gridDim.y) {
     if (op != ASM_RHS && coef[inst].skip) continue;
@@ -391,6 +393,7 @@ __global__ void __launch_bounds__(256) assemble_df_kernel(
 template <typename CT>
 __global__ void force_kernel(const CT *__restrict__ y_in, CT *__restrict__ force, const PhysDev *__restrict__ phys,
                              int K, int batch) {
+  after_previous();
   const int NX = K + 1, NK = 2 * K + 1;
   const size_t spec = (size_t)NK * NK * NX;
   const size_t total = spec * batch;
@@ -415,6 +418,7 @@ __global__ void force_kernel(const CT *__restrict__ y_in, CT *__restrict__ force
 // (a pass of its own, only for instances with the force on), stored as double-float values.
 __global__ void force_dfloat_kernel(const cdf *__restrict__ y_in, cdf *__restrict__ force,
                                     const PhysDev *__restrict__ phys, int K, int batch) {
+  after_previous();
   const int NX = K + 1, NK = 2 * K + 1;
   const size_t spec = (size_t)NK * NK * NX;
   const size_t total = spec * batch;
@@ -580,6 +584,7 @@ __global__ void __launch_bounds__(256, AB2 ? 3 : 2)
                                        const cdf *__restrict__ force, int op_, int stage, int K, int batch,
                                        float inv_n3, FastDiv nx, FastDiv nk) {
   const int op = AB2 ? (int)ASM_AB2 : op_;
+  after_previous();
   const unsigned spec = nk.d * nk.d * nx.d;
   for (int inst = blockIdx.y; inst < batch; inst += gridDim.y) {
     if (op != ASM_RHS && coef[inst].skip) continue;
@@ -596,6 +601,7 @@ __global__ void __launch_bounds__(256, AB2 ? 3 : 2)
 __global__ void step_dt_kernel(unsigned long long *__restrict__ smax_bits, const PhysDev *__restrict__ phys,
                                TimeState *__restrict__ ts, StepCoef *__restrict__ coef, int batch, int n, int K,
                                double dt_fixed, double cfl_adv, double cfl_visc) {
+  after_previous();
   const int inst = blockIdx.x * blockDim.x + threadIdx.x;
   if (inst >= batch) return;
   const double m = __longlong_as_double((long long)smax_bits[inst]);
@@ -747,20 +753,18 @@ cudaError_t launch_assemble(const cplx64 *flux, const cplx64 *y_in, cplx64 *stat
   const double inv_n3 = 0.5 / ((double)d.n * d.n * d.n);
   const AsmGrid g = asm_grid(d);
   const auto kfn = op == ASM_AB2 ? assemble_kernel<cplx64, true> : assemble_kernel<cplx64, false>;
-  kfn<<<g.grid, g.threads, 2 * d.nk * sizeof(double), s>>>(flux, y_in, state, hist, ystage, rhs_out, phys, coef, force,
-                                                           op, stage, d.k, d.batch, inv_n3, fast_div(d.nx),
-                                                           fast_div(d.nk));
-  return cudaGetLastError();
+  return launch_after(kfn, g.grid, dim3(g.threads), 2 * d.nk * sizeof(double), s, flux, y_in, state, hist, ystage,
+                      rhs_out, phys, coef, force, op, stage, d.k, d.batch, inv_n3, fast_div(d.nx), fast_div(d.nk));
 }
 
 cudaError_t launch_force(const cplx64 *y_in, cplx64 *force, const PhysDev *phys, const Dims &d, cudaStream_t s) {
-  force_kernel<cplx64><<<grid_for(d.spec * d.batch, 256), 256, 0, s>>>(y_in, force, phys, d.k, d.batch);
-  return cudaGetLastError();
+  return launch_after(force_kernel<cplx64>, dim3(grid_for(d.spec * d.batch, 256)), dim3(256), 0, s, y_in, force, phys,
+                      d.k, d.batch);
 }
 
 cudaError_t launch_force(const cplx32 *y_in, cplx32 *force, const PhysDev *phys, const Dims &d, cudaStream_t s) {
-  force_kernel<cplx32><<<grid_for(d.spec * d.batch, 256), 256, 0, s>>>(y_in, force, phys, d.k, d.batch);
-  return cudaGetLastError();
+  return launch_after(force_kernel<cplx32>, dim3(grid_for(d.spec * d.batch, 256)), dim3(256), 0, s, y_in, force, phys,
+                      d.k, d.batch);
 }
 
 cudaError_t launch_assemble_df(const cplx32 *flux, const cplx32 *y_in, cplx32 *s_hi, cplx32 *s_lo, cplx32 *hist,
@@ -769,9 +773,8 @@ cudaError_t launch_assemble_df(const cplx32 *flux, const cplx32 *y_in, cplx32 *s
   const float inv_n3 = (float)(0.5 / ((double)d.n * d.n * d.n));  // with the split's 1/2
   const AsmGrid g = asm_grid(d);
   const auto kfn = op == ASM_AB2 ? assemble_df_kernel<true> : assemble_df_kernel<false>;
-  kfn<<<g.grid, g.threads, 0, s>>>(flux, y_in, s_hi, s_lo, hist, ystage, rhs_out, phys, coef, force, op, stage, d.k,
-                                   d.batch, inv_n3, fast_div(d.nx), fast_div(d.nk));
-  return cudaGetLastError();
+  return launch_after(kfn, g.grid, dim3(g.threads), 0, s, flux, y_in, s_hi, s_lo, hist, ystage, rhs_out, phys, coef,
+                      force, op, stage, d.k, d.batch, inv_n3, fast_div(d.nx), fast_div(d.nk));
 }
 
 cudaError_t launch_assemble(const cdf *flux, const cdf *y_in, cdf *state, cdf *hist, cdf *ystage, cplx64 *rhs_out,
@@ -780,14 +783,13 @@ cudaError_t launch_assemble(const cdf *flux, const cdf *y_in, cdf *state, cdf *h
   const float inv_n3 = (float)(0.5 / ((double)d.n * d.n * d.n));  // a power of two, with the split's 1/2
   const AsmGrid g = asm_grid(d);
   const auto kfn = op == ASM_AB2 ? assemble_dfloat_kernel<true> : assemble_dfloat_kernel<false>;
-  kfn<<<g.grid, g.threads, 0, s>>>(flux, y_in, state, hist, ystage, rhs_out, phys, coef, force, op, stage, d.k,
-                                   d.batch, inv_n3, fast_div(d.nx), fast_div(d.nk));
-  return cudaGetLastError();
+  return launch_after(kfn, g.grid, dim3(g.threads), 0, s, flux, y_in, state, hist, ystage, rhs_out, phys, coef, force,
+                      op, stage, d.k, d.batch, inv_n3, fast_div(d.nx), fast_div(d.nk));
 }
 
 cudaError_t launch_force(const cdf *y_in, cdf *force, const PhysDev *phys, const Dims &d, cudaStream_t s) {
-  force_dfloat_kernel<<<grid_for(d.spec * d.batch, 256), 256, 0, s>>>(y_in, force, phys, d.k, d.batch);
-  return cudaGetLastError();
+  return launch_after(force_dfloat_kernel, dim3(grid_for(d.spec * d.batch, 256)), dim3(256), 0, s, y_in, force, phys,
+                      d.k, d.batch);
 }
 
 cudaError_t launch_split_state(const cplx64 *in, cdf *out, size_t count, cudaStream_t s) {
@@ -812,9 +814,8 @@ cudaError_t launch_combine_state(const cplx32 *hi, const cplx32 *lo, cplx64 *out
 
 cudaError_t launch_step_dt(unsigned long long *smax_bits, const PhysDev *phys, TimeState *ts, StepCoef *coef,
                            const Dims &d, double dt_fixed, double cfl_adv, double cfl_visc, cudaStream_t s) {
-  step_dt_kernel<<<(d.batch + 127) / 128, 128, 0, s>>>(smax_bits, phys, ts, coef, d.batch, d.n, d.k, dt_fixed, cfl_adv,
-                                                       cfl_visc);
-  return cudaGetLastError();
+  return launch_after(step_dt_kernel, dim3((d.batch + 127) / 128), dim3(128), 0, s, smax_bits, phys, ts, coef, d.batch,
+                      d.n, d.k, dt_fixed, cfl_adv, cfl_visc);
 }
 
 cudaError_t launch_diag_finish(const double *part, int nparts, const cplx64 *state, const PhysDev *phys,

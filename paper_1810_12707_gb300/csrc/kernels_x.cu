@@ -115,8 +115,8 @@ template <int N, typename C>
 __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restrict__ out,
                                             const PhysDev *__restrict__ phys,
                                             unsigned long long *__restrict__ smax_bits, int K, int blocks_per_inst,
-                                            const typename tw_of<C>::type *__restrict__ tw, typename grid_of<C>::type *__restrict__ bgrid,
-                                            unsigned w, C *sm, double *red) {
+                                            const typename tw_of<C>::type *__restrict__ tw,
+                                            typename grid_of<C>::type *__restrict__ bgrid, unsigned w, C *sm, double *red) {
   constexpr int KT = (N - 1) / 3;  // the 2/3-rule cut-off, fixed by N
   using R = typename C::value_type;
   constexpr int P = pencil_pitch<C>(N);
@@ -315,10 +315,12 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
 template <int N, typename C>
 __global__ void __launch_bounds__((flux_threads<N, C>()), (flux_min_blocks<N, C>()))
     flux_x_kernel(const C *__restrict__ in, C *__restrict__ out, const PhysDev *__restrict__ phys,
-                  unsigned long long *__restrict__ smax_bits, int K, int blocks_per_inst, const typename tw_of<C>::type *__restrict__ tw,
+                  unsigned long long *__restrict__ smax_bits, int K, int blocks_per_inst,
+                  const typename tw_of<C>::type *__restrict__ tw,
                   typename grid_of<C>::type *__restrict__ bgrid) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
+  after_previous();
   flux_x_item<N, C>(in, out, phys, smax_bits, K, blocks_per_inst, tw, bgrid, blockIdx.x,
                     reinterpret_cast<C *>(smem_raw), red);
 }
@@ -555,6 +557,7 @@ __global__ void __launch_bounds__(kXThreads) set_x_kernel(Fields7<const double> 
   constexpr int NX = (N - 1) / 3 + 1, TPP = tpp_for<N, 8>(), P = pencil_pitch<C>(N);
   constexpr size_t NN = (size_t)N * N;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   const int g = threadIdx.x / TPP, t = threadIdx.x - g * TPP;
   const int id = blockIdx.x * x_groups<N>() + g;
   const bool active = id < pencils;
@@ -602,6 +605,7 @@ __global__ void __launch_bounds__(kXThreads) get_x_kernel(const C *__restrict__ 
   constexpr int NX = (N - 1) / 3 + 1, TPP = tpp_for<N, 8>(), P = pencil_pitch<C>(N);
   constexpr size_t NN = (size_t)N * N;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  after_previous();
   const int g = threadIdx.x / TPP, t = threadIdx.x - g * TPP;
   const int id = blockIdx.x * x_groups<N>() + g;
   const bool active = id < pencils;
@@ -728,8 +732,9 @@ __global__ void __launch_bounds__(kDiagThreads) diag_x_kernel(const cplx64 *__re
 namespace {
 
 template <int N, typename C>
-cudaError_t flux_n(const C *in, C *out, const PhysDev *phys, unsigned long long *part, const Dims &d, const typename tw_of<C>::type *tw,
-                   cudaStream_t s, int *err, typename grid_of<C>::type *bgrid, uint32_t wait_polls, unsigned *ctr) {
+cudaError_t flux_n(const C *in, C *out, const PhysDev *phys, unsigned long long *part, const Dims &d,
+                   const typename tw_of<C>::type *tw, cudaStream_t s, int *err, typename grid_of<C>::type *bgrid,
+                   uint32_t wait_polls, unsigned *ctr) {
   constexpr int PAIRS = pairs_for(N);
   if constexpr (PAIRS == 1 && sizeof(C) == 8) {
     if (bgrid != nullptr) err = nullptr;  // the pipelined variant does not write the grid field
@@ -777,8 +782,8 @@ cudaError_t flux_n(const C *in, C *out, const PhysDev *phys, unsigned long long 
     kfn<<<(unsigned)grid, threads, smem, s>>>(in, out, phys, part, d.k, bpi, tw, bgrid, (unsigned)blocks, ctr);
     return cudaGetLastError();
   }
-  flux_x_kernel<N, C><<<(unsigned)blocks, threads, smem, s>>>(in, out, phys, part, d.k, bpi, tw, bgrid);
-  return cudaGetLastError();
+  return launch_after(flux_x_kernel<N, C>, dim3((unsigned)blocks), dim3(threads), smem, s, in, out, phys, part, d.k,
+                      bpi, tw, bgrid);
 }
 
 template <int N, typename C, typename TW>
@@ -789,9 +794,8 @@ cudaError_t set_n(const double *rho, const double *u, const double *b, C *out, c
   if (pencils == 0) return cudaSuccess;
   const unsigned blocks = (unsigned)((pencils + x_groups<N>() - 1) / x_groups<N>());
   const size_t smem = (size_t)x_groups<N>() * pencil_pitch<C>(N) * sizeof(C);  // below 48 KB for every N
-  set_x_kernel<N, C, TW><<<blocks, kXThreads, smem, s>>>(Fields7<const double>{rho, u, b, fstride}, out, tw, row_begin,
-                                                         (int)pencils);
-  return cudaGetLastError();
+  return launch_after(set_x_kernel<N, C, TW>, dim3(blocks), dim3(kXThreads), smem, s,
+                      Fields7<const double>{rho, u, b, fstride}, out, tw, row_begin, (int)pencils);
 }
 
 template <int N, typename C>
@@ -802,9 +806,8 @@ cudaError_t get_n(const C *in, double *a, double *b, double *c, int nf, const Di
   if (pencils == 0) return cudaSuccess;
   const unsigned blocks = (unsigned)((pencils + x_groups<N>() - 1) / x_groups<N>());
   const size_t smem = (size_t)x_groups<N>() * pencil_pitch<C>(N) * sizeof(C);
-  get_x_kernel<N, C><<<blocks, kXThreads, smem, s>>>(in, Fields7<double>{a, b, c, fstride}, nf, tw, row_begin,
-                                                     (int)pencils);
-  return cudaGetLastError();
+  return launch_after(get_x_kernel<N, C>, dim3(blocks), dim3(kXThreads), smem, s, in, Fields7<double>{a, b, c, fstride},
+                      nf, tw, row_begin, (int)pencils);
 }
 
 template <int N>

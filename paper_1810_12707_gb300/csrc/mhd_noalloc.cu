@@ -107,9 +107,11 @@ cudaError_t setup_device(unsigned char **base) {
   return cudaSuccess;
 }
 
-// The instance's parameters, written on the caller's stream from kernel arguments.
-__global__ void set_phys_kernel(mhd::PhysDev *pd, double nu, double eta, double cs) {
+// The instance's parameters, written on the caller's stream from kernel arguments, and the word the
+// flux pass takes its atomic maximum on (and screens against), cleared.
+__global__ void set_phys_kernel(mhd::PhysDev *pd, double nu, double eta, double cs, unsigned long long *word) {
   *pd = mhd::make_phys(nu, eta, cs);
+  *word = 0ull;
 }
 
 }  // namespace
@@ -138,10 +140,8 @@ extern "C" MHD_API mhd_status mhd_rhs_noalloc(int32_t n, const mhd_phys *phys, c
   double *part = reinterpret_cast<double *>(base + kOffPart);
   const mhd::TwFx *tw = reinterpret_cast<const mhd::TwFx *>(base + (n == 16 ? kOffTw16 : kOffTw32));
   mhd::PhysDev *pd = reinterpret_cast<mhd::PhysDev *>(base + kOffPhys);
-  set_phys_kernel<<<1, 1, 0, s>>>(pd, phys->nu, phys->eta, phys->cs);
+  set_phys_kernel<<<1, 1, 0, s>>>(pd, phys->nu, phys->eta, phys->cs, reinterpret_cast<unsigned long long *>(part));
   NA_CK(cudaGetLastError());
-  // the flux pass takes an atomic maximum here (and screens against it): start from zero
-  NA_CK(cudaMemsetAsync(part, 0, sizeof(unsigned long long), s));
 
   // state spectra from the real-space fields (m = rho u), truncated and normalised
   const size_t n3 = (size_t)n * n * n;
