@@ -7,8 +7,8 @@
 // rows (inverse x), divides, and sends u back (forward x); the y and z column passes then give the
 // truncated spectrum u_hat.  A mode k belongs to shell s = round(|k|), decided exactly in integer
 // arithmetic: (2s - 1)^2 <= 4|k|^2 < (2s + 1)^2 (|k|^2 is an integer, so no mode lies on a shell
-// boundary).  A shell's blocks walk every (k_z, k_y) row of the truncated half spectrum, find the k_x
-// run of the shell, and sum in a fixed order, so the spectra are bitwise reproducible.
+// boundary).  Warps walk the rows of the truncated half spectrum and add each shell's run of k_x to
+// their own bins in a fixed order, so the spectra are bitwise reproducible.
 #include "fft_device.cuh"
 #include "fp64_util.cuh"
 #include "launch_util.cuh"
@@ -96,64 +96,97 @@ __device__ __forceinline__ double curl_dot(double kx, double ky, double kz, cplx
   return (fx.im * tx.re - fx.re * tx.im) + (fy.im * ty.re - fy.re * ty.im) + (fz.im * tz.re - fz.re * tz.im);
 }
 
-// Block (s, c): shell s, rows of chunk c (of gridDim.y).  uh, bh: 3 truncated spectra each (stride
-// `spec`); out[c][s][5] =
+// Shell sums.  uh, bh: 3 truncated spectra each (stride `spec`); per shell s the five sums
 // (sum w |u_hat|^2 / 2, sum w |B_hat|^2 / 2, sum w |k . u_hat|^2, sum w Re(conj(u_hat) . i k x u_hat),
-// sum w Re(conj(B_hat) . i k x B_hat) / |k|^2) over the shell, with w = 1 on the k_x = 0 plane and 2
-// elsewhere (the half spectrum stands for k and -k).  By Parseval the last two are the shell's
-// shares of the kinetic helicity <u . curl u> and of the magnetic helicity <A . B>, A_hat =
-// i k x B_hat / |k|^2 (Coulomb gauge, A_hat(0) = 0).  dh = i k_x u_hat_x and gh = i k . B_hat on
-// every mode (each mode is visited by exactly one block).  The chunks' sums are added in order.
-// One block per shell left the outer shells' blocks to finish alone: 256^3 3.62 -> 1.43 ms.
-__global__ void __launch_bounds__(256) shell_kernel(const cplx64 *__restrict__ uh, const cplx64 *__restrict__ bh,
-                                                    cplx64 *__restrict__ dh, cplx64 *__restrict__ gh,
-                                                    double *__restrict__ out, int K) {
-  __shared__ double red[32];
+// sum w Re(conj(B_hat) . i k x B_hat) / |k|^2), with w = 1 on the k_x = 0 plane and 2 elsewhere (the
+// half spectrum stands for k and -k).  By Parseval the last two are the shell's shares of the kinetic
+// helicity <u . curl u> and of the magnetic helicity <A . B>, A_hat = i k x B_hat / |k|^2 (Coulomb
+// gauge, A_hat(0) = 0).  dh = i k_x u_hat_x and gh = i k . B_hat on every mode.
+// A warp takes 32 consecutive k_x of one (k_z, k_y) row, so that every lane has a mode and the FP64
+// pipe, which bounds this, works on full warps; along a row the shells come in order, so each
+// shell's lanes are a run whose sums one lane per quantity adds up from shared memory into the warp's
+// own bins.  The warps' rows, the runs and the blocks' sums are added in a fixed order.  A thread per
+// row and shell, the earlier form, kept a quarter of its lanes busy: 256^3 1.43 -> 0.545 ms.
+constexpr int kShellWarps = 4;
+__global__ void __launch_bounds__(32 * kShellWarps) shell_kernel(const cplx64 *__restrict__ uh,
+                                                                 const cplx64 *__restrict__ bh,
+                                                                 cplx64 *__restrict__ dh, cplx64 *__restrict__ gh,
+                                                                 double *__restrict__ part, int K, int ns) {
+  extern __shared__ double shell_sm[];  // [warp][5 ns] bins, [warp][32][5] terms
+  __shared__ int shell_of[kShellWarps][32];
   const int NX = K + 1, NK = 2 * K + 1;
   const size_t spec = (size_t)NK * NK * NX;
-  const int s = blockIdx.x;
-  const long long lo_b = s == 0 ? 0 : (long long)(2 * s - 1) * (2 * s - 1);
-  const long long hi_b = (long long)(2 * s + 1) * (2 * s + 1);
-  double ek = 0.0, em = 0.0, th = 0.0, hk = 0.0, hm = 0.0;
-  for (int r = blockIdx.y * blockDim.x + threadIdx.x; r < NK * NK; r += gridDim.y * blockDim.x) {
-    const int kz = kept_wave(r / NK, K), ky = kept_wave(r % NK, K);
-    const long long q4 = 4LL * (ky * ky + kz * kz);
-    if (q4 >= hi_b) continue;
-    int kx = 0;
-    if (q4 < lo_b) {
-      kx = (int)(0.5f * sqrtf((float)(lo_b - q4)));  // within 1; made exact in integers
-      while (kx > 0 && q4 + 4LL * (kx - 1) * (kx - 1) >= lo_b) --kx;
-      while (q4 + 4LL * kx * kx < lo_b) ++kx;
-    }
-    for (; kx <= K && q4 + 4LL * kx * kx < hi_b; ++kx) {
-      const size_t m = (size_t)r * NX + kx;
-      const double w = kx == 0 ? 1.0 : 2.0;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double *bins = shell_sm + (size_t)warp * 5 * ns;
+  double *term = shell_sm + (size_t)kShellWarps * 5 * ns + warp * 160;
+  for (int i = lane; i < 5 * ns; i += 32) bins[i] = 0.0;
+  __syncwarp();
+  const int chunks = (NX + 31) / 32, items = NK * NK * chunks;
+  for (int it = blockIdx.x * kShellWarps + warp; it < items; it += gridDim.x * kShellWarps) {
+    const int r = it / chunks, kxi = (it - r * chunks) * 32 + lane;
+    const int kzi = kept_wave(r / NK, K), kyi = kept_wave(r % NK, K);
+    const bool valid = kxi <= K;
+    const int k2 = kxi * kxi + kyi * kyi + kzi * kzi;
+    // round(|k|): the integer s with (2s - 1)^2 <= 4 |k|^2 < (2s + 1)^2
+    int s = (int)(sqrtf((float)k2) + 0.5f);
+    while ((2 * s + 1) * (2 * s + 1) <= 4 * k2) ++s;
+    while (s > 0 && (2 * s - 1) * (2 * s - 1) > 4 * k2) --s;
+    if (valid) {
+      const size_t m = (size_t)r * NX + kxi;
+      const double kx = kxi, ky = kyi, kz = kzi;
+      const double w = kxi == 0 ? 1.0 : 2.0;
       const cplx64 ux = uh[m], uy = uh[spec + m], uz = uh[2 * spec + m];
       const cplx64 bx = bh[m], by = bh[spec + m], bz = bh[2 * spec + m];
-      ek += w * 0.5 * (ux.re * ux.re + ux.im * ux.im + uy.re * uy.re + uy.im * uy.im + uz.re * uz.re + uz.im * uz.im);
-      em += w * 0.5 * (bx.re * bx.re + bx.im * bx.im + by.re * by.re + by.im * by.im + bz.re * bz.re + bz.im * bz.im);
+      double *e = term + 5 * lane;
+      e[0] = 0.5 * w * (ux.re * ux.re + ux.im * ux.im + uy.re * uy.re + uy.im * uy.im + uz.re * uz.re + uz.im * uz.im);
+      e[1] = 0.5 * w * (bx.re * bx.re + bx.im * bx.im + by.re * by.re + by.im * by.im + bz.re * bz.re + bz.im * bz.im);
       const double dr = kx * ux.re + ky * uy.re + kz * uz.re, di = kx * ux.im + ky * uy.im + kz * uz.im;
-      th += w * (dr * dr + di * di);
+      e[2] = w * (dr * dr + di * di);
       dh[m] = cplx64{-kx * ux.im, kx * ux.re};
-      hk += w * curl_dot(kx, ky, kz, ux, uy, uz);
-      const long long k2 = (long long)kx * kx + (long long)ky * ky + (long long)kz * kz;
-      if (k2 > 0) hm += w * curl_dot(kx, ky, kz, bx, by, bz) / (double)k2;
+      e[3] = w * curl_dot(kx, ky, kz, ux, uy, uz);
+      const double k2d = k2 > 0 ? (double)k2 : 1.0, c = w * curl_dot(kx, ky, kz, bx, by, bz);
+      e[4] = k2 > 0 ? quotient(c, k2d, rcp3(k2d)) : 0.0;
       const double gr = kx * bx.re + ky * by.re + kz * bz.re, gi = kx * bx.im + ky * by.im + kz * bz.im;
       gh[m] = cplx64{-gi, gr};
     }
+    shell_of[warp][lane] = s;
+    const int before = __shfl_up_sync(0xffffffffu, s, 1);
+    const unsigned heads = __ballot_sync(0xffffffffu, valid && (lane == 0 || s != before));
+    const int count = __popc(__ballot_sync(0xffffffffu, valid));
+    __syncwarp();
+    const int runs = __popc(heads);
+    for (int i = lane; i < 5 * runs; i += 32) {
+      const int j = i / 5, q = i - 5 * j;
+      const int first = __fns(heads, 0, j + 1), end = j + 1 < runs ? (int)__fns(heads, 0, j + 2) : count;
+      double v = term[5 * first + q];
+      for (int l = first + 1; l < end; ++l) v += term[5 * l + q];
+      bins[5 * shell_of[warp][first] + q] += v;
+    }
+    __syncwarp();
   }
-  const double a = block_sum(ek, red);
-  const double b = block_sum(em, red);
-  const double c = block_sum(th, red);
-  const double e = block_sum(hk, red);
-  const double f = block_sum(hm, red);
-  if (threadIdx.x == 0) {
-    double *o = out + 5 * ((size_t)blockIdx.y * gridDim.x + s);
-    o[0] = a;
-    o[1] = b;
-    o[2] = c;
-    o[3] = e;
-    o[4] = f;
+  __syncthreads();
+  for (int i = threadIdx.x; i < 5 * ns; i += blockDim.x) {
+    double v = shell_sm[i];
+#pragma unroll
+    for (int w = 1; w < kShellWarps; ++w) v += shell_sm[(size_t)w * 5 * ns + i];
+    part[(size_t)blockIdx.x * 5 * ns + i] = v;
+  }
+}
+
+// out[i] = sum over the blocks of part[block][i], i < n: 32 sums per block, 8 threads each, in a fixed
+// order.
+__global__ void __launch_bounds__(256) shell_sum_kernel(const double *__restrict__ part, int blocks, int n,
+                                                        double *__restrict__ out) {
+  __shared__ double red[8][32];
+  const int l = threadIdx.x & 31, w = threadIdx.x >> 5, i = blockIdx.x * 32 + l;
+  double v = 0.0;
+  if (i < n)
+    for (int b = w; b < blocks; b += 8) v += part[(size_t)b * n + i];
+  red[w][l] = v;
+  __syncthreads();
+  if (w == 0 && i < n) {
+    for (int k = 1; k < 8; ++k) v += red[k][l];
+    out[i] = v;
   }
 }
 
@@ -230,9 +263,18 @@ cudaError_t launch_velocity_x(const cplx64 *in, cplx64 *out, const Dims &d, cons
   }
 }
 
-cudaError_t launch_shells(const cplx64 *uh, const cplx64 *bh, cplx64 *dh, cplx64 *gh, double *out, const Dims &d,
-                          int chunks, cudaStream_t s) {
-  shell_kernel<<<dim3(num_shells(d.k), chunks), 256, 0, s>>>(uh, bh, dh, gh, out, d.k);
+cudaError_t launch_shells(const cplx64 *uh, const cplx64 *bh, cplx64 *dh, cplx64 *gh, double *part, int blocks,
+                          const Dims &d, cudaStream_t s) {
+  const int ns = num_shells(d.k), n = 5 * ns;
+  const size_t smem = (size_t)kShellWarps * (n + 160) * sizeof(double);
+  if (smem > 48 * 1024) {
+    cudaError_t e = ensure_smem<shell_kernel>((int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  shell_kernel<<<blocks, 32 * kShellWarps, smem, s>>>(uh, bh, dh, gh, part + n, d.k, ns);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  shell_sum_kernel<<<(n + 31) / 32, 256, 0, s>>>(part + n, blocks, n, part);
   return cudaGetLastError();
 }
 

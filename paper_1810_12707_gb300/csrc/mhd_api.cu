@@ -1362,7 +1362,7 @@ mhd_status mhd_spectra(mhd_ctx *c, int32_t inst, double *ek, double *em, int32_t
   const size_t n3 = (size_t)d.n * d.n * d.n;
   const size_t part_len = sizes_for(c->d, c->precision).part;
   const int mblocks = (int)std::min<size_t>(2 * 152, part_len / 2);
-  if ((size_t)5 * ns > part_len || mblocks < 1) return fail(c, MHD_EINVAL, "scratch too small for the spectra");
+  if (mblocks < 1) return fail(c, MHD_EINVAL, "scratch too small for the spectra");
   const cplx64 *Si = nullptr;
   if ((st = state_fp64(c, inst, &Si))) return st;
   // u_hat: inverse z, y of the state; u = m / rho with the x passes; forward y, z
@@ -1374,11 +1374,13 @@ mhd_status mhd_spectra(mhd_ctx *c, int32_t inst, double *ek, double *em, int32_t
   // (clear of u_hat, 3 spec values, and of all that the du_x/dx chain below writes into W1: its
   // z-pass output and n^3 real values; W1 holds at least 7 n^3 doubles)
   cplx64 *gh = c->W1 + n3;
-  // blocks per shell: as many as the partials' buffer holds sums of, at most 32
-  const int chunks = (int)std::min<size_t>(32, part_len / ((size_t)5 * ns));
-  CK(mhd::launch_shells(c->W1, Si + 4 * d.spec, c->W2, gh, c->part, d, chunks, c->stream));
-  std::vector<double> sh((size_t)5 * ns * chunks);
-  CK(cudaMemcpyAsync(sh.data(), c->part, sh.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  // the shells' sums go behind the du_x/dx spectrum in W2 (7 n^2 (K + 1) complex values hold both for
+  // every n): at most 305 sums of 5 ns doubles
+  const int sblocks = (int)std::min<size_t>(2 * 152, ((size_t)d.nk * d.nk * ((d.nx + 31) / 32) + 3) / 4);
+  double *spart = reinterpret_cast<double *>(c->W2 + d.spec);
+  CK(mhd::launch_shells(c->W1, Si + 4 * d.spec, c->W2, gh, spart, sblocks, d, c->stream));
+  std::vector<double> sh((size_t)5 * ns);
+  CK(cudaMemcpyAsync(sh.data(), spart, sh.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   // du_x/dx on the grid, then its moments
   CK(mhd::launch_col_inverse(c->W2, c->W1, d.n, 1, d.nk * d.nx, c->tw, c->stream));
@@ -1398,8 +1400,6 @@ mhd_status mhd_spectra(mhd_ctx *c, int32_t inst, double *ek, double *em, int32_t
   CK(cudaMemcpyAsync(ap.data(), c->part, ap.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   double th = 0.0, m2 = 0.0, m3 = 0.0, hk = 0.0, hm = 0.0, dmax = 0.0;
-  for (size_t i = 0; i < (size_t)5 * ns; ++i)
-    for (int q = 1; q < chunks; ++q) sh[i] += sh[(size_t)q * 5 * ns + i];
   for (int s = 0; s < ns; ++s) {
     if (ek) ek[s] = sh[5 * s];
     if (em) em[s] = sh[5 * s + 1];

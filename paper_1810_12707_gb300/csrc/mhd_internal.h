@@ -305,14 +305,15 @@ cudaError_t launch_assemble_iz(const cplx32 *flux, cplx32 *s_hi, cplx32 *s_lo, c
 // Final reduction of the diagnostic partials of one instance plus the spectral terms; writes
 // 24 doubles to `out` (see mhd_api.cu for the order).
 // Shell spectra (kernels_spectra.cu).  launch_velocity_x: rho, m (fields 0..3 of [7][z][y][kx],
-// one instance) -> u = m / rho -> forward x -> [3][z][y][kx].  launch_shells: `chunks` blocks
-// per shell, out[chunk][s][5] = (E_u, E_B, sum |k.u_hat|^2, kinetic helicity, magnetic helicity) of shell s,
-// dh = i k_x u_hat_x and gh = i k . B_hat on every kept mode.  launch_moments: part[b][2] =
+// one instance) -> u = m / rho -> forward x -> [3][z][y][kx].  launch_shells: part[s][5] =
+// (E_u, E_B, sum |k.u_hat|^2, kinetic helicity, magnetic helicity) of shell s, from the sums of
+// `blocks` blocks left behind them (part holds (blocks + 1) 5 num_shells doubles); dh = i k_x u_hat_x
+// and gh = i k . B_hat on every kept mode.  launch_moments: part[b][2] =
 // (sum v^2, sum v^3) of a fixed share of v; launch_absmax: part[b] = max |v| of a fixed share.
 int num_shells(int k);
 cudaError_t launch_velocity_x(const cplx64 *in, cplx64 *out, const Dims &d, const TwFx *tw, cudaStream_t s);
-cudaError_t launch_shells(const cplx64 *uh, const cplx64 *bh, cplx64 *dh, cplx64 *gh, double *out, const Dims &d,
-                          int chunks, cudaStream_t s);
+cudaError_t launch_shells(const cplx64 *uh, const cplx64 *bh, cplx64 *dh, cplx64 *gh, double *part, int blocks,
+                          const Dims &d, cudaStream_t s);
 cudaError_t launch_moments(const double *v, size_t n, double *part, int blocks, cudaStream_t s);
 cudaError_t launch_absmax(const double *v, size_t n, double *part, int blocks, cudaStream_t s);
 
