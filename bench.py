@@ -235,18 +235,13 @@ KERNEL_SOURCES = {
     "flux_x": ("kernels_x.cu", "fft_device.cuh", "fixed64.cuh"),
     "col": ("kernels_col.cu", "fft_device.cuh", "fixed64.cuh"),
 }
+_CAPTURE = "ncu dram__bytes metrics on one launch of this size (one pass), profiles/ncu_kernels_256.md"
 TRAFFIC = {
     # (kernel, n, batch, precision): (bytes per launch, source hash, capture)
-    ("flux_x", 256, 1, "fp64"): (634_281_728 + 1_029_447_000, "8098a458af43095a",
-                                 "ncu --set full, profiles/ncu_flux_x_abc256_fp64.md"),
-    ("flux_x", 256, 1, "fp32"): (315_693_312 + 489_866_752, "8098a458af43095a",
-                                 "ncu --set full, profiles/ncu_abc256_fp32.md"),
-    ("flux_x", 256, 1, "fp64df"): (631_424_000 + 1_028_800_512, "76c413daf911ef3f",
-                                   "ncu --set full, profiles/ncu_df_kernels_abc256.md"),
-    # the 512^3 launch, captured directly with these three metrics (one ncu pass, so nothing is
-    # saved or restored around it), profiles/ncu_df_kernels_abc256.md
-    ("flux_x", 512, 1, "fp64df"): (5_023_917_824 + 8_550_996_480, "76c413daf911ef3f",
-                                   "ncu dram__bytes metrics on one 512^3 launch, profiles/ncu_df_kernels_abc256.md"),
+    ("flux_x", 256, 1, "fp64"): (631_834_112 + 1_027_939_584, "4cf5be480dcce365", _CAPTURE),
+    ("flux_x", 256, 1, "fp32"): (315_802_880 + 487_820_288, "4cf5be480dcce365", _CAPTURE),
+    ("flux_x", 256, 1, "fp64df"): (631_350_528 + 1_029_372_928, "4cf5be480dcce365", _CAPTURE),
+    ("flux_x", 512, 1, "fp64df"): (5_022_098_688 + 8_562_965_760, "4cf5be480dcce365", _CAPTURE),
 }
 
 
