@@ -656,6 +656,12 @@ mhd_status get_state_staged(mhd_ctx *c, const C *src, const typename mhd::tw_of<
   return MHD_OK;
 }
 
+// Waits for the copies of earlier asynchronous gets into their callers' buffers.
+mhd_status async_gets_done(mhd_ctx *c) {
+  if (c->out_stream) CK(cudaStreamSynchronize(c->out_stream));
+  return MHD_OK;
+}
+
 // Truncated spectra `src` of one instance -> host rho, m, B through the staging slots in W1.
 // MHD_EINVAL (nothing queued) when no staging plan fits.
 template <typename C>
@@ -664,7 +670,6 @@ mhd_status get_state_host(mhd_ctx *c, const C *src, const typename mhd::tw_of<C>
   if (!slab_plan(c, &pl)) return MHD_EINVAL;
   mhd_status st = ensure_copy_stream(c);
   if (st) return st;
-  if (c->out_stream) CK(cudaStreamSynchronize(c->out_stream));  // an earlier asynchronous get
   // two slots: more measured slower for the synchronous transfer out
   const Staging sg = {pl.dz, 2, {pl.slot[0], pl.slot[1]}, c->copy_stream, c->ev_full, c->ev_free};
   return get_state_staged(c, src, tw, rho, m, b, sg, true);
@@ -746,11 +751,8 @@ mhd_status mhd_set_state(mhd_ctx *c, int32_t inst, const double *rho, const doub
   return MHD_OK;
 }
 
-mhd_status mhd_get_state(mhd_ctx *c, int32_t inst, double *rho, double *m, double *b, int32_t on_device) {
-  mhd_status st = check_inst(c, inst);
-  if (st) return st;
-  if (!rho || !m || !b) return fail(c, MHD_EINVAL, "null output");
-  DeviceGuard g(c);
+static mhd_status get_state(mhd_ctx *c, int32_t inst, double *rho, double *m, double *b, int32_t on_device) {
+  mhd_status st;
   if (c->precision == MHD_FP64_DF) {
     // double-float transforms straight from the double-float state
     const cdf *Sd = statedf(c, inst);
@@ -765,6 +767,22 @@ mhd_status mhd_get_state(mhd_ctx *c, int32_t inst, double *rho, double *m, doubl
   if ((st = state_fp64(c, inst, &src))) return st;
   if (!on_device && (st = get_state_host(c, src, c->tw, rho, m, b)) != MHD_EINVAL) return st;
   return spectra_to_real(c, src, rho, m, b, on_device);
+}
+
+mhd_status mhd_get_state(mhd_ctx *c, int32_t inst, double *rho, double *m, double *b, int32_t on_device) {
+  mhd_status st = check_inst(c, inst);
+  if (st) return st;
+  if (!rho || !m || !b) return fail(c, MHD_EINVAL, "null output");
+  DeviceGuard g(c);
+  // The buffers of earlier asynchronous gets are filled when this returns, whichever path it takes.
+  // Host outputs may be those very buffers, so those copies end first; they overlap a device get.
+  if (!on_device && (st = async_gets_done(c))) return st;
+  st = get_state(c, inst, rho, m, b, on_device);
+  if (on_device) {
+    const mhd_status done = async_gets_done(c);
+    if (!st) st = done;
+  }
+  return st;
 }
 
 mhd_status mhd_get_state_async(mhd_ctx *c, int32_t inst, double *rho, double *m, double *b) {
