@@ -298,21 +298,22 @@ mhd_status copy_out(mhd_ctx *c, void *dst, const void *src, size_t bytes, int on
   return MHD_OK;
 }
 
-// The inverse x pass of the 7 fields in W2 into rho/m/B outputs: straight into device arrays, through
-// W1 to the host.  Synchronises.
+// The inverse x pass of the 7 fields in W2 into rho/m/B outputs: straight into arrays of the context's
+// GPU, through W1 and copies to the host and to any other device array.  Synchronises.
 template <typename C>
 mhd_status rows_out(mhd_ctx *c, const C *w2, const typename mhd::tw_of<C>::type *tw, double *a, double *b3, double *c3,
                     int on_device) {
   const size_t n3 = (size_t)c->d.n * c->d.n * c->d.n;
-  if (on_device) {
+  if (on_device && mhd::direct_output(a, c->device) && mhd::direct_output(b3, c->device) &&
+      mhd::direct_output(c3, c->device)) {
     CK(mhd::launch_get_x(w2, a, b3, c3, one(c), tw, c->stream));
   } else {
     mhd_status st;
     double *real = reinterpret_cast<double *>(c->W1);
     CK(mhd::launch_get_x(w2, real, real + n3, real + 4 * n3, one(c), tw, c->stream));
-    if ((st = copy_out(c, a, real, n3 * sizeof(double), 0))) return st;
-    if ((st = copy_out(c, b3, real + n3, 3 * n3 * sizeof(double), 0))) return st;
-    if ((st = copy_out(c, c3, real + 4 * n3, 3 * n3 * sizeof(double), 0))) return st;
+    if ((st = copy_out(c, a, real, n3 * sizeof(double), on_device))) return st;
+    if ((st = copy_out(c, b3, real + n3, 3 * n3 * sizeof(double), on_device))) return st;
+    if ((st = copy_out(c, c3, real + 4 * n3, 3 * n3 * sizeof(double), on_device))) return st;
   }
   CK(cudaStreamSynchronize(c->stream));
   return MHD_OK;

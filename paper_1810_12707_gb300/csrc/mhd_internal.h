@@ -23,6 +23,22 @@
 
 namespace mhd {
 
+// Whether kernels of GPU `device` may store doubles straight into a caller's array at p: memory of
+// that GPU (type and owner as cudaPointerGetAttributes gives them) at a double's alignment.  All else
+// that cudaMemcpyAsync writes to -- another GPU's memory, page-locked or managed memory, an odd
+// address -- takes the results by a copy.
+inline bool direct_output(int type, int owner, int device, const void *p) {
+  return type == (int)cudaMemoryTypeDevice && owner == device && (uintptr_t)p % sizeof(double) == 0;
+}
+inline bool direct_output(const void *p, int device) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return direct_output((int)a.type, a.device, device, p);
+}
+
 constexpr int kStateFields = 7;  // rho, m_x, m_y, m_z, B_x, B_y, B_z
 constexpr int kFluxFields = 12;  // T_xx T_yy T_zz T_xy T_xz T_yz, E_x E_y E_z, u_x u_y u_z
 

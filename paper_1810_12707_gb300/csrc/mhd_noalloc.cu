@@ -159,6 +159,16 @@ extern "C" MHD_API mhd_status mhd_rhs_noalloc(int32_t n, const mhd_phys *phys, c
   NA_CK(mhd::launch_assemble(W1, S, S, nullptr, nullptr, R, pd, nullptr, mhd::ASM_RHS, 0, d, s));
   NA_CK(mhd::launch_col_inverse(R, W1, n, 7, d.nk * d.nx, tw, s));
   NA_CK(mhd::launch_col_inverse(W1, W2, n, 7 * n, d.nx, tw, s));
-  NA_CK(mhd::launch_get_x(W2, drho, dm, db, d, tw, s));
+  int dev = 0;
+  NA_CK(cudaGetDevice(&dev));
+  if (mhd::direct_output(drho, dev) && mhd::direct_output(dm, dev) && mhd::direct_output(db, dev)) {
+    NA_CK(mhd::launch_get_x(W2, drho, dm, db, d, tw, s));
+    return MHD_OK;
+  }
+  double *real = reinterpret_cast<double *>(W1);
+  NA_CK(mhd::launch_get_x(W2, real, 7, d, tw, s));
+  NA_CK(cudaMemcpyAsync(drho, real, n3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
+  NA_CK(cudaMemcpyAsync(dm, real + n3, 3 * n3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
+  NA_CK(cudaMemcpyAsync(db, real + 4 * n3, 3 * n3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
   return MHD_OK;
 }
