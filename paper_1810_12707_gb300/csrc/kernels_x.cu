@@ -14,6 +14,7 @@
 // brought to the grid, the 12 products of the RHS are formed pointwise in shared memory (no
 // real-space array ever reaches HBM), and their forward transforms leave as truncated half
 // spectra.  Rows are indexed r = z*N + y; a block owns PAIRS consecutive row pairs.
+#include "cfl_screen.cuh"
 #include "fft_device.cuh"
 #include "fp64_util.cuh"
 #include "launch_util.cuh"
@@ -71,14 +72,6 @@ constexpr int flux_min_blocks() {
 // 512^3 20.5 -> 19.8, but 256^3 2.31 -> 2.33).
 template <int N, typename C>
 constexpr bool flux_ahead() { return std::is_same<C, cplx64>::value ? N != 512 : !std::is_same<C, cdf>::value; }
-
-// |x| as an FP32 number from the high word alone, truncated (at most 2^-20 relative below |x|);
-// infinite from 2^128 on and for a NaN, 0 below 2^-126.  Integer instructions: a conversion costs
-// as much as an FP64 multiplication.
-__device__ __forceinline__ float float_below(double x) {
-  const int h = (__double2hiint(x) & 0x7fffffff) - 0x38000000;
-  return __int_as_float(min(max(h, 0), 0x0ff00000) << 3);
-}
 
 // Run the FFT of `np` pencils (pencil id -> shared-memory pointer `ptr(id)`) with every group of
 // N/VPT threads of the block taking one pencil at a time.  Each pencil is touched by its group only,
@@ -161,17 +154,11 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
   constexpr bool kDF = std::is_same<C, cdf>::value;
   using SM = typename std::conditional<kDF, double, R>::type;  // type of the CFL maximum
   SM smax = 0;
-  // FP64 and double-float: the maximum that blocks of this pass have already published is a
-  // lower bound of the pass's maximum.  A point whose FP32 estimate of |u| + c_f lies below
-  // `screen` (that bound less 3e-6 relative and 1e-18 absolute, above the estimate's worst error:
-  // 3e-7 relative from FP32 sums and roots, and in FP64 1e-6 from the truncated operands) cannot
-  // raise it, so its exact speed (two FP64 square roots) is not formed.  The pass still yields the
-  // exact maximum, whichever blocks ran first; a NaN, an infinite estimate or a negative density
-  // always takes the exact path.
+  // FP64 and double-float: exact speeds only where they can raise the published maximum
   float screen = 0.f;
   if constexpr (sizeof(SM) == 8) {
     const double lb = __longlong_as_double((long long)*reinterpret_cast<volatile unsigned long long *>(smax_bits + inst));
-    screen = (float)(lb * (1.0 - 3e-6) - 1e-18);
+    screen = cfl_screen(lb);
   }
   if constexpr (kDF) {
     // double-float products.  The grid values leave the inverse transforms unnormalised; near a
@@ -225,8 +212,7 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
         bd[2 * 9 * P + h] = ux;
         bd[2 * 10 * P + h] = uy;
         bd[2 * 11 * P + h] = uz;
-        const float u2f = ux.hi * ux.hi + uy.hi * uy.hi + uz.hi * uz.hi, c2f = cs2.hi + b2.hi * ir.hi;
-        if (!(sqrtf(u2f) + sqrtf(c2f) < screen)) {
+        if (cfl_may_raise(ux.hi, uy.hi, uz.hi, cs2.hi, b2.hi, ir.hi, screen)) {
           const dfr nx = dfr_norm(ux), ny = dfr_norm(uy), nz = dfr_norm(uz);
           const dfr u2 = dfr_norm(nx * nx + ny * ny + nz * nz), c2 = dfr_norm(cs2 + b2 * ir);
           const double s = sqrt(dfr_to_double(u2)) + sqrt(dfr_to_double(c2));
@@ -282,9 +268,7 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
       bd[2 * 10 * P + h] = uy;
       bd[2 * 11 * P + h] = uz;
       if constexpr (sizeof(R) == 8) {
-        const float fx = float_below(ux), fy = float_below(uy), fz = float_below(uz);
-        const float u2f = fx * fx + fy * fy + fz * fz, c2f = cs2f + float_below(b2) * float_below(ir);
-        if (!(sqrtf(u2f) + sqrtf(c2f) < screen) || __double2hiint(ir) < 0) {
+        if (cfl_may_raise(ux, uy, uz, cs2f, b2, ir, screen)) {
           const R s = sqrt(ux * ux + uy * uy + uz * uz) + sqrt(cs2 + b2 * ir);
           smax = (s != s || s > smax) ? s : smax;  // keeps a NaN once seen
         }
