@@ -591,6 +591,9 @@ __device__ __forceinline__ void stockham_stages(C *buf, int t, bool active, cons
   }
 }
 
+// The rest of a `bad` pencil's result.
+__device__ __forceinline__ void fx_bad_out(cplx64 &x, const FxScale &sc) { x = c_scale(x, fx_bad_factor(sc.ek)); }
+
 // ---- The FP64 pencil FFT (fixed64.cuh) ----
 // The same Stockham stages on a pencil of doubles.  The first stage reads doubles, finds the
 // pencil's common exponent and converts; the pencil is fixed-point complex values between the
@@ -652,10 +655,14 @@ __device__ __forceinline__ void fx_stages(cfx *buf, int t, bool active, const Tw
           cplx64 d;
           if constexpr (DP) d = cplx64{fx_to_double_dp(x.re, be), fx_to_double_dp(x.im, be)};
           else d = cplx64{fx_to_double(x.re, be), fx_to_double(x.im, be)};
-          if (sc.bad) d.re = d.im = fx_double(0x7ff80000u, 0u);
           *reinterpret_cast<cplx64 *>(p) = d;
         }
       }
+    }
+    if (NS * R == N && sc.bad) {
+      cplx64 *pen = reinterpret_cast<cplx64 *>(buf);
+#pragma unroll 1
+      for (int i = t; i < N; i += TPP) fx_bad_out(pen[sm_at<cplx64>((unsigned)i)], sc);
     }
   }
   group_sync<TPP>();
@@ -698,7 +705,7 @@ __device__ __forceinline__ FxScale fx_group_scale(uint32_t m, Size size) {
 #pragma unroll
     for (int i = 1; i < TPP / 32; ++i) p = fx_merge(p, part[w0 + i]);
   }
-  return fx_scale(p, LOG2G);
+  return fx_scale_any(p, LOG2G);
 }
 
 // The transform of the doubles x[r] = element t + r N/8 of each thread of the group: results in the
@@ -718,7 +725,7 @@ __device__ __forceinline__ void fx_fft_from(const cplx64 *x, cplx64 *buf, int t,
     if (ZP && (r == 3 || r == 4)) continue;
     m = max(m, max(fx_hi(x[r].re) & 0x7fffffffu, fx_hi(x[r].im) & 0x7fffffffu));
   }
-  const FxScale sc = fx_group_scale<N, true>(m >> 20, [&](uint32_t mm) {
+  const FxScale sc = fx_group_scale<N, true>(fx_max_exp(m), [&](uint32_t mm) {
     uint32_t a = 0u;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
@@ -730,11 +737,18 @@ __device__ __forceinline__ void fx_fft_from(const cplx64 *x, cplx64 *buf, int t,
   cfx *fb = reinterpret_cast<cfx *>(buf);
   if (active) {
     cfx v[8];
+    if (!sc.bad) {
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      if (ZP && (r == 3 || r == 4)) continue;
-      v[r] = cfx{fx_from_double(fx_hi(x[r].re), fx_lo(x[r].re), sc.ek),
-                 fx_from_double(fx_hi(x[r].im), fx_lo(x[r].im), sc.ek)};
+      for (int r = 0; r < 8; ++r) {
+        if (ZP && (r == 3 || r == 4)) continue;
+        v[r] = cfx{fx_from_double(fx_hi(x[r].re), fx_lo(x[r].re), sc.ek),
+                   fx_from_double(fx_hi(x[r].im), fx_lo(x[r].im), sc.ek)};
+      }
+    } else {
+      const uint32_t ek = fx_bad_ek(sc.ek);
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        v[r] = cfx{fx_from_any(fx_hi(x[r].re), fx_lo(x[r].re), ek), fx_from_any(fx_hi(x[r].im), fx_lo(x[r].im), ek)};
     }
     fx_dft8<DIR, ZP>(v);
 #pragma unroll
@@ -853,7 +867,7 @@ __device__ __forceinline__ void rows_inverse(C *buf, int t, bool active, RowPair
       m = max(m, max(fx_hi(x.x1[i].re) & 0x7fffffffu, fx_hi(x.x1[i].im) & 0x7fffffffu));
     }
     // a thread's values bound its own inputs of the first stage and their mirror images alike
-    const FxScale sc = fx_group_scale<N, false>(m >> 20, [&](uint32_t mm) {
+    const FxScale sc = fx_group_scale<N, false>(fx_max_exp(m), [&](uint32_t mm) {
       uint32_t a = 0u;
 #pragma unroll
       for (int i = 0; i < NI; ++i)
@@ -863,14 +877,19 @@ __device__ __forceinline__ void rows_inverse(C *buf, int t, bool active, RowPair
     });
     cfx *fb = reinterpret_cast<cfx *>(buf);
     cfx v[8];
-#pragma unroll
-    for (int i = 0; i < NI; ++i) {
-      const int64_t a = fx_from_double(fx_hi(x.x0[i].re), fx_lo(x.x0[i].re), sc.ek);
-      const int64_t b = fx_from_double(fx_hi(x.x0[i].im), fx_lo(x.x0[i].im), sc.ek);
-      const int64_t c = fx_from_double(fx_hi(x.x1[i].re), fx_lo(x.x1[i].re), sc.ek);
-      const int64_t d = fx_from_double(fx_hi(x.x1[i].im), fx_lo(x.x1[i].im), sc.ek);
+    auto pack = [&](int i, int64_t a, int64_t b, int64_t c, int64_t d) {
       v[i] = cfx{a - d, b + c};
       if (active && RP::kept(t, i) && (i > 0 || t > 0)) *RP::mirror(fb, t, i) = cfx{a + d, c - b};
+    };
+    if (!sc.bad) {
+      auto fx = [&](double y) { return fx_from_double(fx_hi(y), fx_lo(y), sc.ek); };
+#pragma unroll
+      for (int i = 0; i < NI; ++i) pack(i, fx(x.x0[i].re), fx(x.x0[i].im), fx(x.x1[i].re), fx(x.x1[i].im));
+    } else {
+      const uint32_t ek = fx_bad_ek(sc.ek);
+      auto fx = [&](double y) { return fx_from_any(fx_hi(y), fx_lo(y), ek); };
+#pragma unroll
+      for (int i = 0; i < NI; ++i) pack(i, fx(x.x0[i].re), fx(x.x0[i].im), fx(x.x1[i].re), fx(x.x1[i].im));
     }
     group_sync<TPP>();
     if (active) {
@@ -949,13 +968,21 @@ __device__ __forceinline__ void rows_split(E *z, const FxScale &sc, C *buf, int 
         auto out = [&](int64_t v) { return DP ? fx_to_double_dp(v, be) : fx_to_double(v, be); };
         y0 = C{out(r0.re), out(r0.im)};
         y1 = C{out(r1.re), out(r1.im)};
-        if (sc.bad) y0.re = y0.im = y1.re = y1.im = fx_double(0x7ff80000u, 0u);
       } else {
         y0 = post(r0);
         y1 = post(r1);
       }
       dst[t + i * TPP] = y0;
       dst[NX + t + i * TPP] = y1;
+    }
+    if constexpr (kFx) {
+      if (sc.bad) {
+#pragma unroll 1
+        for (int k = t; k < NX; k += TPP) {
+          fx_bad_out(dst[k], sc);
+          fx_bad_out(dst[NX + k], sc);
+        }
+      }
     }
   }
 }

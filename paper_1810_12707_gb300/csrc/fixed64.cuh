@@ -16,8 +16,9 @@
 // where an FP64 butterfly rounds at 2^-53 of its values.  Values more than 2^60 below the largest
 // first-stage sum round to zero; in FP64 they are lost in the same butterflies' rounding errors.
 //
-// A pencil with a NaN or an infinity (or a magnitude above 2^976) transforms to NaN everywhere;
-// one whose largest magnitude is below 2^-959 transforms to zeros.
+// A pencil with a NaN or an infinity transforms to NaN everywhere.  The conversions that every pencil
+// takes hold for largest magnitudes from 2^-959 to 2^977; any other takes the paths of FxScale::bad,
+// which hold over the whole range of doubles (but a pencil below 2^-1042 altogether is taken as zeros).
 #pragma once
 
 #include <stdint.h>
@@ -117,6 +118,12 @@ FX_FN uint32_t fx_exp(uint32_t hi) { return (hi >> 20) & 0x7ffu; }
 FX_FN uint32_t fx_size(uint32_t hi, uint32_t m) {
   return fx_shr((hi & 0xfffffu) | 0x100000u, m - fx_exp(hi)) + 1u;
 }
+// The biased exponent of the largest of some magnitudes, from the largest of their high words: 1 if
+// they are all subnormal, 0 if all zero.
+FX_FN uint32_t fx_max_exp(uint32_t hi) {
+  const uint32_t e = hi >> 20, any = hi < 1u ? hi : 1u;
+  return e > any ? e : any;
+}
 // What some of a pencil's values say: the largest biased exponent m, the largest first-stage sum a
 // and the whole sum t / 8, both in units of 2^(m - 1043).
 struct FxPart {
@@ -148,6 +155,24 @@ FX_FN FxScale fx_scale(FxPart p, int log2_groups) {
   s.bad = p.m >= 2000u;
   return s;
 }
+// The scale of any pencil.  `bad`: outside the range of the conversions that the transforms use (and
+// not all zeros, which those handle).  Such a pencil's `ek` is moved by 256 towards the middle: its
+// values are converted by fx_from_any with fx_bad_ek, its results as ever and then multiplied by
+// fx_bad_factor, 2^-256, 2^256 or NaN.  Both sit behind branches that a whole group takes or not, the
+// multiplications in loops: as predicated instructions in line they held the FP64 pipe in every pencil
+// (256^3 FP64 run 140 -> 159 ms; so, 138 ms).
+FX_FN FxScale fx_scale_any(FxPart p, int log2_groups) {
+  const bool low = p.m - 1u < 63u, out = low || p.m >= 2000u;
+  FxPart q = p;
+  if (out) q.m = low ? p.m + 256u : p.m == 2047u ? 4096u : p.m - 256u;
+  FxScale s = fx_scale(q, log2_groups);
+  s.bad = out;
+  return s;
+}
+FX_FN uint32_t fx_bad_ek(uint32_t ek) { return ek < 1024u ? ek - 256u : ek + 256u; }
+FX_FN double fx_bad_factor(uint32_t ek) {
+  return fx_double(ek >= 4096u ? 0x7ff80000u : ek < 1024u ? 0x2ff00000u : 0x4ff00000u, 0u);
+}
 
 // ---- conversions ----
 FX_FN int64_t fx_from_double(uint32_t hi, uint32_t lo, uint32_t ek) {
@@ -156,6 +181,14 @@ FX_FN int64_t fx_from_double(uint32_t hi, uint32_t lo, uint32_t ek) {
   const uint32_t h = (mh << 10) | (lo >> 22), l = lo << 10;
   const uint32_t s2 = s > 32u ? s - 32u : 0u;
   const int64_t v = fx_join(fx_shr(h, s), fx_shr(fx_funnel_r(l, h, s), s2));
+  return (int32_t)hi < 0 ? -v : v;
+}
+// The same for every exponent: subnormal numbers have no leading one, and zero is zero.
+FX_FN int64_t fx_from_any(uint32_t hi, uint32_t lo, uint32_t ek) {
+  const uint32_t e = fx_exp(hi), s = ek - (e ? e : 1u);
+  const uint32_t mh = (hi & 0xfffffu) | (e ? 0x100000u : 0u);
+  const uint64_t m = (((uint64_t)mh << 32) | lo) << 10;
+  const int64_t v = s > 63u ? 0 : (int64_t)(m >> s);
   return (int32_t)hi < 0 ? -v : v;
 }
 // v 2^(be - 1086), rounded to nearest (`be`: the biased exponent of a value whose leading one is

@@ -609,13 +609,19 @@ __global__ void __launch_bounds__(kXThreads) get_x_kernel(const C *__restrict__ 
         const uint32_t be = sc.ek + (uint32_t)sc.shift + 1u;
         v0 = fx_to_double_dp(z[r].re, be);
         v1 = fx_to_double_dp(z[r].im, be);
-        if (sc.bad) v0 = v1 = fx_double(0x7ff80000u, 0u);
       } else {
         v0 = x_store(z[r].re);
         v1 = x_store(z[r].im);
       }
       dst[r * TPP] = v0;
       dst[N + r * TPP] = v1;
+    }
+    if constexpr (std::is_same<C, cplx64>::value) {
+      if (sc.bad) {
+        const double f = fx_bad_factor(sc.ek);
+#pragma unroll 1
+        for (int r = 0; r < 16; ++r) dst[r * TPP] *= f;  // N = 8 TPP: both rows
+      }
     }
   }
 }
