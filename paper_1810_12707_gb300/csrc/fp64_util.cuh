@@ -26,10 +26,12 @@ __device__ __forceinline__ bool rcp3_covers(double x) {
 }
 // m / x with r = 1 / x from rcp3: the quotient m r corrected by its remainder (Markstein), which
 // rounds correctly but for rare cases (|m| above 2^-960, or the remainder may be subnormal).  Three
-// instructions.
+// instructions.  An infinite m r is the quotient: its remainder would be infinite too, and their sum a
+// NaN.
 __device__ __forceinline__ double quotient(double m, double x, double r) {
   const double q = m * r;
-  return fma(fma(-x, q, m), r, q);
+  const double c = fma(fma(-x, q, m), r, q);
+  return (__double2hiint(q) & 0x7ff00000) == 0x7ff00000 ? q : c;
 }
 
 // sqrt(x) = s (1 + e/2 + 3 e^2 / 8), s = x y, e = 1 - s^2 / x, y the approximate 1 / sqrt(x): the

@@ -74,6 +74,14 @@ def test_quotient(run):
     assert max(ulps(v, Fraction(float(a)) / Fraction(float(b))) for v, a, b in zip(q, m, x)) <= 0.5 + 2.0 ** -10
 
 
+def test_quotient_outside_the_range(run):
+    x = np.array([2.0 ** -600, -2.0 ** -600, 0.3, -0.3, 0.3, 1.7, 1.7, 2.0 ** 900])
+    m = np.array([2.0 ** 600, 2.0 ** 600, np.inf, np.inf, -np.inf, np.nan, 0.0, 2.0 ** -900])
+    q = run(QUOTIENT, m, x)
+    with np.errstate(all="ignore"):
+        assert np.array_equal(q, m / x, equal_nan=True)
+
+
 def test_square_root(run):
     x = np.abs(np.concatenate([numbers(11, 12000, -1022, 1023), numbers(12, 4000, -2, 2),
                                [2.0 ** -1022, 2.0 ** -959, np.nextafter(2.0 ** -959, 0), np.finfo(float).max]]))
