@@ -24,6 +24,11 @@ __device__ __forceinline__ bool rcp3_covers(double x) {
   const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu;
   return h - 0x00200000u < 0x7fa00000u;
 }
+// 1 / x for every x: the flux pass's, whose densities may be anything.
+__device__ __forceinline__ double rcp_any(double x) {
+  if (rcp3_covers(x)) return rcp3(x);
+  return 1.0 / x;
+}
 // m / x with r = 1 / x from rcp3: the quotient m r corrected by its remainder (Markstein), which
 // rounds correctly but for rare cases (|m| above 2^-960, or the remainder may be subnormal).  Three
 // instructions.  An infinite m r is the quotient: its remainder would be infinite too, and their sum a

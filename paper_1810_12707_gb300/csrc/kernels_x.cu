@@ -249,7 +249,7 @@ __device__ __forceinline__ void flux_x_item(const C *__restrict__ in, C *__restr
       const R mx = v[h][1], my = v[h][2], mz = v[h][3];
       const R bx = v[h][4], by = v[h][5], bz = v[h][6];
       R ir;
-      if constexpr (sizeof(R) == 8) ir = rcp3(rho);
+      if constexpr (sizeof(R) == 8) ir = rcp_any(rho);
       else ir = (R)1 / rho;
       const R ux = mx * ir, uy = my * ir, uz = mz * ir;
       const R b2 = bx * bx + by * by + bz * bz;

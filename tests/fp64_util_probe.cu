@@ -8,6 +8,7 @@ __global__ void probe(int which, int n, const double *a, const double *b, double
   if (which == 1) out[i] = mhd::quotient(a[i], b[i], mhd::rcp3(b[i]));
   if (which == 2) out[i] = mhd::sqrt3(a[i]);
   if (which == 3) out[i] = mhd::rcp3_covers(a[i]) ? 1.0 : 0.0;
+  if (which == 4) out[i] = mhd::rcp_any(a[i]);
 }
 
 // Returns the CUDA status (0: success).

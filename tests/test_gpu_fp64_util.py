@@ -21,7 +21,7 @@ pytestmark = pytest.mark.gpu
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_1810_12707_gb300", "csrc")
 NVCC = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
-RCP, QUOTIENT, SQRT, COVERS = range(4)
+RCP, QUOTIENT, SQRT, COVERS, RCP_ANY = range(5)
 
 
 @pytest.fixture(scope="module")
@@ -58,10 +58,11 @@ def ulps(value, exact):
     return abs(Fraction(float(value)) - exact) / Fraction(math.ulp(float(exact)))
 
 
-def test_reciprocal(run):
+@pytest.mark.parametrize("which", [RCP, RCP_ANY])
+def test_reciprocal(run, which):
     x = np.concatenate([numbers(1, 12000, -1021, 1020), numbers(2, 4000, -3, 3),
                         [2.0 ** -1021, -2.0 ** -1021, np.nextafter(2.0 ** 1021, 0)]])
-    r = run(RCP, x)
+    r = run(which, x)
     assert max(ulps(v, 1 / Fraction(float(a))) for v, a in zip(r, x)) <= 0.5 + 2.0 ** -4
 
 
@@ -105,3 +106,5 @@ def test_the_range_of_the_reciprocal(run):
     x = np.concatenate([x, -x])
     expected = (np.abs(x) >= edges[0]) & (np.abs(x) < edges[1])
     assert np.array_equal(run(COVERS, x) == 1.0, expected)
+    with np.errstate(all="ignore"):  # outside it the general reciprocal divides
+        assert np.array_equal(run(RCP_ANY, x[~expected]), 1.0 / x[~expected], equal_nan=True)
