@@ -169,8 +169,8 @@ MHD_API mhd_status mhd_get_state(mhd_ctx *ctx, int32_t inst, double *rho, double
  * (mhd_get_state and mhd_destroy also wait for them).  The first call allocates its staging,
  * kept until mhd_destroy: the whole state, 7 N^3 doubles (about 36 % of mhd_footprint_bytes of
  * one instance), when that is at most half of mhd_footprint_bytes, else fewer slabs of N/8
- * z-planes (at least two, then thinner ones; up to 128^3 one slab of all planes).  Errors: MHD_EINVAL (bad instance, null buffer),
- * MHD_ENOMEM (staging), MHD_ECUDA. */
+ * z-planes (at least two, then thinner ones; up to 128^3 one slab of all planes).  Errors:
+ * MHD_EINVAL (bad instance, null buffer), MHD_ENOMEM (staging), MHD_ECUDA. */
 MHD_API mhd_status mhd_get_state_async(mhd_ctx *ctx, int32_t inst, double *rho, double *m, double *b);
 
 /* Real-space right-hand side of instance `inst` at its current state (the inverse transform of

@@ -12,8 +12,10 @@
 // are bounded by A, the largest sum of |re| + |im| over one butterfly's inputs, the transform by
 // T, the sum over the whole pencil.  The inputs are converted so that A fills 60 bits, and the
 // stages after the first shift right only as far as T / A demands (the shift rides on the
-// twiddles), so the unit of the fixed-point numbers is at most about 2^-56 of the result's RMS,
-// where an FP64 butterfly rounds at 2^-53 of its values.  Values more than 2^60 below the largest
+// twiddles), so the unit of the fixed-point numbers is at most 2^-59 T.  T is at most sqrt(2 N) of the
+// result's RMS (Parseval; all magnitudes equal): the unit is at most 2^-56 of the RMS at 32 points,
+// 2^-54 at 512, 2^-53.5 at 1024, and far less for spectra with a few large modes; an FP64
+// butterfly rounds every value of every stage at 2^-53.  Values more than 2^60 below the largest
 // first-stage sum round to zero; in FP64 they are lost in the same butterflies' rounding errors.
 //
 // A pencil with a NaN or an infinity transforms to NaN everywhere.  The conversions that every pencil

@@ -479,8 +479,8 @@ struct SlabPlan {
 // pageable memory 71 / 952; 64^3 135 / 475, 159 / 1039; 128^3 759 / 868, 6425 / 40569.
 constexpr int kHostPieceMaxN = 128;
 
-// As many slots of N/8 z-planes as W1 holds behind the y-pass output, up to one per slab (so
-// that a transfer in can run ahead of the transforms); thinner slabs when not even two fit.
+// Above it: as many slots of N/8 z-planes as W1 holds behind the y-pass output, up to one per slab
+// (so that a transfer in can run ahead of the transforms); thinner slabs when not even two fit.
 bool slab_plan(mhd_ctx *c, SlabPlan *pl) {
   const mhd::Dims &d = c->d;
   if (d.n <= kHostPieceMaxN) return false;
@@ -560,11 +560,11 @@ mhd_status set_state_host(mhd_ctx *c, const double *rho, const double *u, const 
   return MHD_OK;
 }
 
-// Staging of a device-to-host transfer: two slots of 7 x dz N^2 doubles, the stream that copies
+// Staging of a device-to-host transfer: slots of 7 x dz N^2 doubles, the stream that copies
 // out of them and the events that hand them between that stream and the context's stream.
 struct Staging {
   int dz;
-  int ns;  // slots, 2..8, used in turn
+  int ns;  // slots, 1..8, used in turn
   double *slot[8];
   cudaStream_t cs;
   cudaEvent_t *full, *free;
@@ -573,7 +573,7 @@ struct Staging {
 // The staging of mhd_get_state_async, allocated on first use: slots of N/8 z-planes, as many as
 // there are slabs (8: the whole state, so that the transforms never wait for the copies out) when
 // that takes at most half the context's footprint (it takes about 36 % at every N), else fewer (at
-// least 2, then thinner slabs).
+// least 2, then thinner slabs); up to kHostPieceMaxN one slot of all planes.
 mhd_status async_staging(mhd_ctx *c, Staging *sg) {
   const size_t n = c->d.n, nn = n * n;
   if (!c->out_stream) {
