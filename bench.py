@@ -5,9 +5,9 @@ Default workload (`--config tg512`): N = 512^3 Taylor-Green flow u = (sin x cos 
 -cos x sin y cos z, 0) with a seeded random |k| <= 4 magnetic field at <|B|^2>/2 = 1e-3 (seed 2),
 Mach 0.3, nu = eta = 1e-3, rho0 = 1, CFL-limited dt, in the FP64-tolerance double-float mode
 (MHD_FP64_DF: every value a pair of FP32 numbers, 48-bit significand; parity with the FP64 oracle
-to <= 1e-10 after 100 steps).  The same line carries, as extra keys, the same workload in IEEE
-FP64 and in the FP32 mixed mode with each mode's relative L2 error per field against IEEE FP64
-after 100 steps, the plain cuFFT build at 512^3 FP64, and a short served segment of the serving
+to <= 1e-10 after 100 steps).  The same line carries, as extra keys, the same workload in MHD_FP64
+(IEEE data and grid products, transforms in 64-bit fixed point) and in the FP32 mixed mode with each
+mode's relative L2 error per field against MHD_FP64 after 100 steps, the plain cuFFT build at 512^3 FP64, and a short served segment of the serving
 configuration (Poisson requests N in {32, 64, 128, 256}) with p50/p99 latencies.  Other
 configurations: `abc256` (256^3 ABC dynamo, FP64), `ot32` (Orszag-Tang type, 32^3 FP64, fixed dt
 1e-3), `ens64` (64 independent 64^3 Orszag-Tang instances, mixed precision, one batched launch
@@ -58,6 +58,7 @@ def paper_baseline(n: int):
     return {256: PAPER_256_V100, 512: PAPER_512_P100}.get(n)
 FP32_PEAK_TFLOPS = 80.5   # 152 SMs x 128 FP32 FMA/clk x 2 flop x 2.07 GHz
 FP32_PEAK_TOPS = 40.27    # FP32 lane operations per second: 152 SMs x 128 lanes x 2.07 GHz (x 1e12)
+FP64_SLOTS = 64           # of these lane operations' time that one FP64 instruction takes (2 per clock and SM)
 ORACLE_MAX_N = 256        # largest grid the oracle is timed on (about 16 GB of host memory)
 
 CONFIGS = {
@@ -136,10 +137,10 @@ def kernel_model(n: int, batch: int = 1, precision: str = "fp64"):
         ops = dfloat_ops(n)
         m = {key: (b, ops[key]) for key, (b, f) in m.items()}
     elif precision == "fp64":
-        # the FP64 passes transform in 64-bit fixed point: "flops" become the instructions per lane
-        # that the method needs (fixed_ops)
+        # the FP64 passes transform in 64-bit fixed point: "flops" become the lane slots that the
+        # method takes on the busier of its two pipes (fixed_ops)
         ops = fixed_ops(n)
-        m = {key: (b, ops[key]) for key, (b, f) in m.items()}
+        m = {key: (b, ops[key][0]) for key, (b, f) in m.items()}
     return {key: (b * batch, f * batch) for key, (b, f) in m.items()}
 
 
@@ -192,7 +193,8 @@ def fixed_fft_ops(n: int) -> float:
     the stages of dfloat_fft_ops with a complex sum 4 (two 32-bit halves of two parts), a complex
     twiddle product 38 (12 multiplications of 32 x 32 bits, 26 splits, shifts and sums), a product by
     sqrt(2)/2 10; and per value the conversion in 40 (exponent, size and shifts of two parts) and out
-    6 (two additions of the FP64 pipe and one integer instruction a part)."""
+    6 (two additions of the FP64 pipe and one integer instruction a part; about 20 integer ones a part
+    where they run on the integer pipe)."""
     stages, rem = 0, n
     while rem >= 8:
         rem //= 8
@@ -207,24 +209,27 @@ def fixed_fft_ops(n: int) -> float:
 
 
 def fixed_ops(n: int) -> dict:
-    """Instructions per lane and launch of each FP64 kernel (one instance): transforms
-    (fixed_fft_ops), the grid products (about 30 FP64 and 40 other instructions per grid value) and the
-    spectral assembly with the update (about 90 FP64 and 60 others per mode).  An FP64 instruction
-    takes 75 of these slots' time on its own pipe; the figure counts it once."""
+    """(lane slots, pipe) per launch of each FP64 kernel (one instance): the larger of its instructions
+    per lane ("issue") and of FP64_SLOTS times those that run on the FP64 pipe ("fp64").  The column
+    passes' FP64 instructions are the conversions of the kept results (2 a part), the flux pass's the
+    grid products (about 30 FP64 and 40 other instructions per grid value; its conversions, about 40
+    instructions a complex value, run on the integer pipe), the assembly's its arithmetic (about 90 FP64 and 60 others per mode)."""
     k = (n - 1) // 3
     nx, nk = k + 1, 2 * k + 1
     spec = nk * nk * nx
     f = fixed_fft_ops(n)
-    return {
-        "inverse_z": 7 * nk * nx * f,
-        "inverse_y": 7 * n * nx * f,
-        "flux_x": (n * n / 2) * (19 * f + 2 * n * 70.0),
-        "step_dt": 0.0,
-        "forward_y": 12 * n * nx * f,
-        "forward_z": 12 * nk * nx * f,
-        "assemble_ab2": 150.0 * spec,
-        "assemble_iz": 150.0 * spec + 7 * nk * nx * f,
+    counts = {  # (instructions, of these FP64)
+        "inverse_z": (7 * nk * nx * f, 7 * nk * nx * n * 4.0),
+        "inverse_y": (7 * n * nx * f, 7 * n * nx * n * 4.0),
+        "flux_x": ((n * n / 2) * (7 * (f + n * 34.0) + 12 * (f - n * 6.0 + 2 * nx * 40.0) + 2 * n * 70.0),
+                   n ** 3 * 30.0),
+        "step_dt": (0.0, 0.0),
+        "forward_y": (12 * n * nx * f, 12 * n * nx * nk * 4.0),
+        "forward_z": (12 * nk * nx * f, 12 * nk * nx * nk * 4.0),
+        "assemble_ab2": (150.0 * spec, 90.0 * spec),
+        "assemble_iz": (150.0 * spec + 7 * nk * nx * f, 90.0 * spec + 7 * nk * nx * n * 4.0),
     }
+    return {key: max((i, "issue"), (FP64_SLOTS * d, "fp64")) for key, (i, d) in counts.items()}
 
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch, from one ncu capture
@@ -232,7 +237,7 @@ def fixed_ops(n: int) -> dict:
 # kernel are the ones it was taken on: the entry keeps a hash of those files and is dropped
 # (traffic reported as null) as soon as they change.
 KERNEL_SOURCES = {
-    "flux_x": ("kernels_x.cu", "fft_device.cuh", "fixed64.cuh"),
+    "flux_x": ("kernels_x.cu", "fft_device.cuh", "fixed64.cuh", "fp64_util.cuh", "cfl_screen.cuh"),
     "col": ("kernels_col.cu", "fft_device.cuh", "fixed64.cuh"),
 }
 _CAPTURE = "ncu dram__bytes metrics on one launch of this size (one pass), profiles/ncu_kernels_256.md"
@@ -565,8 +570,9 @@ def run_ours(args, name, cfg):
             unit, src = ("T FP32-ops/s", "FP32 lanes x clock: 152 SMs x 128 x 2.07 GHz (one operation per lane "
                          "per clock; the algorithmic count is the double-float method's FP32 operations)")
         elif prec == mhd.MHD_FP64:
-            unit, src = ("T instructions/s", "issue slots x lanes x clock: 152 SMs x 128 x 2.07 GHz (the count is the "
-                         "fixed-point method's instructions per lane)")
+            unit, src = ("T lane slots/s", "lanes x clock: 152 SMs x 128 x 2.07 GHz (the count is the fixed-point "
+                         f"method's on its busier pipe, here {fixed_ops(n)[top][1]}: instructions per lane, or "
+                         f"{FP64_SLOTS} per FP64 instruction, of which an SM takes 2 a clock)")
         else:
             unit, src = "TFLOP/s", "FP32 FMA units x clock (probe 74.4 TFLOP/s)"
         roof = {"bound": "alu", "achieved": per[top]["tflops"], "peak": alu_peak, "unit": unit,
@@ -617,9 +623,9 @@ def run_ours(args, name, cfg):
 
 
 def precision_study(cfg, ics, tuned, steps: int = 100, timed: int = 10):
-    """The same workload in IEEE FP64, double-float and mixed precision: device time per step
+    """The same workload in MHD_FP64, double-float and mixed precision: device time per step
     (`timed` graph-replayed steps after 3 warm-up steps, inside the first `steps`), and each mode's
-    relative L2 error per field (rho; m and B as vectors) against IEEE FP64 after `steps` steps,
+    relative L2 error per field (rho; m and B as vectors) against MHD_FP64 after `steps` steps,
     computed on the device."""
     import torch
     from paper_1810_12707_gb300 import mhd
