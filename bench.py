@@ -243,10 +243,10 @@ KERNEL_SOURCES = {
 _CAPTURE = "ncu dram__bytes metrics on one launch of this size (one pass), profiles/ncu_kernels_256.md"
 TRAFFIC = {
     # (kernel, n, batch, precision): (bytes per launch, source hash, capture)
-    ("flux_x", 256, 1, "fp64"): (631_834_112 + 1_027_939_584, "4cf5be480dcce365", _CAPTURE),
-    ("flux_x", 256, 1, "fp32"): (315_802_880 + 487_820_288, "4cf5be480dcce365", _CAPTURE),
-    ("flux_x", 256, 1, "fp64df"): (631_350_528 + 1_029_372_928, "4cf5be480dcce365", _CAPTURE),
-    ("flux_x", 512, 1, "fp64df"): (5_022_098_688 + 8_562_965_760, "4cf5be480dcce365", _CAPTURE),
+    ("flux_x", 256, 1, "fp64"): (631_461_376 + 1_026_626_048, "a2159fc5c32f3407", _CAPTURE),
+    ("flux_x", 256, 1, "fp32"): (315_668_736 + 487_595_520, "a2159fc5c32f3407", _CAPTURE),
+    ("flux_x", 256, 1, "fp64df"): (631_375_872 + 1_027_729_152, "a2159fc5c32f3407", _CAPTURE),
+    ("flux_x", 512, 1, "fp64df"): (5_021_925_120 + 8_562_340_096, "a2159fc5c32f3407", _CAPTURE),
 }
 
 

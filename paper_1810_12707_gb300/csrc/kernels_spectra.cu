@@ -32,7 +32,7 @@ constexpr int threads_for(int tpp, int pencils) {
 
 // rho, m (fields 0..3 of `in`, [f][z][y][kx <= K] after the inverse y pass) -> u = m / rho on the
 // grid -> forward x -> out [3][z][y][kx <= K].  Two real rows per complex pencil, as in the flux
-// pass; a block owns PAIRS row pairs (256^3 1.39 -> 0.82 ms with the rows straight from and to their
+// pass; a block owns PAIRS row pairs (256^3 1.39 -> 0.90 ms with the rows straight from and to their
 // spectra and corrected quotients for the divisions).
 template <int N>
 __global__ void __launch_bounds__(kMaxThreads) velocity_x_kernel(const cplx64 *__restrict__ in,

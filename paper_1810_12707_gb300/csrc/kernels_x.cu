@@ -69,7 +69,7 @@ constexpr int flux_min_blocks() {
 
 // Whether a group loads its next row pair before it transforms one: not where the registers that
 // holds cost more than the loads' latency (double-float 256^3 1.85 -> 1.81 ms, 512^3 17.6 -> 16.4; FP64
-// 512^3 20.5 -> 19.8, but 256^3 2.31 -> 2.33).
+// 512^3 20.5 -> 19.8, but 256^3 2.31 -> 2.33; not compared at 1024^3).
 template <int N, typename C>
 constexpr bool flux_ahead() { return std::is_same<C, cplx64>::value ? N != 512 : !std::is_same<C, cdf>::value; }
 
@@ -632,7 +632,7 @@ __global__ void __launch_bounds__(kXThreads) get_x_kernel(const C *__restrict__ 
 // A block owns PAIRS row pairs and one group per pencil (7 PAIRS of them) where 448 threads hold them.
 // The sums' constant factors are applied once per thread.  Bound by the FP64 pipe: per point one
 // reciprocal, three corrected quotients, three roots, a logarithm and about 20 more instructions
-// (fp64_util.cuh; 256^3 7.15 -> 3.84 ms against divisions, library roots and 7 pencils on 6 groups).
+// (fp64_util.cuh; 256^3 7.15 -> 3.96 ms against divisions, library roots and 7 pencils on 6 groups).
 constexpr int kDiagThreads = 448;
 template <int N>
 __global__ void __launch_bounds__(kDiagThreads) diag_x_kernel(const cplx64 *__restrict__ in,
